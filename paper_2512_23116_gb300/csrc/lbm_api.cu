@@ -22,6 +22,7 @@
 #include "lbm_check.cuh"
 #include "lbm_internal.h"
 #include "lbm_kernels.h"
+#include "lbm_struct.h"
 
 #define LBM_API extern "C" __attribute__((visibility("default")))
 
@@ -437,7 +438,8 @@ int check_err(lbm_t h) {
   CK(h, cudaMemcpyAsync(&e, h->d_err, sizeof e, cudaMemcpyDeviceToHost, h->stream));
   CK(h, cudaStreamSynchronize(h->stream));
   if (kBoundsCheck) {
-    const uint32_t b = bounds_word_tma() | bounds_word_direct() | bounds_word_aux() | bounds_word_random();
+    const uint32_t b = bounds_word_tma() | bounds_word_direct() | bounds_word_aux() | bounds_word_random() |
+                       bounds_word_struct();
     if (b) return fail(h, LBM_ERR_CUDA, "device bounds check failed (checked build; word %u)", b);
   }
   if (e) {
@@ -1216,22 +1218,27 @@ LBM_API int lbm_stats(lbm_t h, int32_t inst, int32_t what, lbm_stats_t* out) {
     if ((int)rs.size() > LBM_MAX_R) rs.resize(LBM_MAX_R);
     out->nr = 0;
     if (rs.empty()) return LBM_OK;
-    const int blocks = std::min(2 * h->num_sms, 1024);
-    const size_t need = ((size_t)blocks + 1) * 6 * rs.size();
+    // every separation in one launch into a [blocks][nr x 6] table, one column
+    // sum, one read-back; separations are at most half the smallest extent
+    // (<= 2^10 cells on a lattice of 2^33), which always fits a tile
+    const int cols = 6 * (int)rs.size();
+    StructPlan plan;
+    cudaError_t pe;
+    if (!plan_struct(p.nx, p.ny, p.nz, rs.data(), (int)rs.size(), false, 4096, &plan, &pe))
+      return fail(h, LBM_ERR_CUDA, "structure functions: %s", cudaGetErrorString(pe));
+    const size_t need = ((size_t)plan.grid + 1) * cols;
     if (need > h->spec_elems) {
       if (h->d_spec) cudaFree(h->d_spec);
       h->d_spec = nullptr;
+      h->spec_elems = 0;
       CK(h, cudaMalloc(&h->d_spec, need * sizeof(double)));
       h->spec_elems = need;
     }
     out->nr = (int)rs.size();
-    // every separation in one launch into a [blocks][nr x 6] table, one column
-    // sum, one read-back
-    const int cols = 6 * (int)rs.size();
-    CK(h, launch_struct_multi(I.u, p.nx, p.ny, p.nz, rs.data(), (int)rs.size(), h->d_spec, blocks, h->stream));
-    CK(h, launch_sum_cols(h->d_spec, blocks, cols, h->d_spec + (size_t)blocks * cols, h->stream));
+    CK(h, launch_struct_plan(I.u, plan, false, h->d_spec, h->stream));
+    CK(h, launch_sum_cols(h->d_spec, plan.grid, cols, h->d_spec + (size_t)plan.grid * cols, h->stream));
     std::vector<double> sp(cols);
-    CK(h, cudaMemcpyAsync(sp.data(), h->d_spec + (size_t)blocks * cols, sizeof(double) * cols,
+    CK(h, cudaMemcpyAsync(sp.data(), h->d_spec + (size_t)plan.grid * cols, sizeof(double) * cols,
                           cudaMemcpyDeviceToHost, h->stream));
     CK(h, cudaStreamSynchronize(h->stream));
     for (size_t k = 0; k < rs.size(); ++k) {

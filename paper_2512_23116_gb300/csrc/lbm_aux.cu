@@ -1,6 +1,6 @@
 // Auxiliary kernels: initial equilibrium, canonical population access in the
-// AA layout, parity re-layout, the FP64 reduction finisher, the shell binning
-// of the energy spectrum and the structure-function reductions.
+// AA layout, parity re-layout, the FP64 reduction finishers and the shell
+// binning of the energy spectrum.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -259,9 +259,10 @@ __global__ void k_spec_bin(const float2* __restrict__ c, int nx, int ny, int nz,
     partials[(int64_t)blockIdx.x * (kmax + 1) + s] += sh[s];
 }
 
-// Column sums of a [rows][cols] table, one warp per column in the fixed order
+// Column sums of a [rows][cols] table times `scale`, one warp per column in the fixed order
 // of k_finish (lane l adds rows l, l + 32, ...; then a shuffle tree).
-__global__ void k_sum_cols(const double* __restrict__ p, int rows, int cols, double* __restrict__ out) {
+__global__ void k_sum_cols(const double* __restrict__ p, int rows, int cols, double scale,
+                           double* __restrict__ out) {
   const int lane = threadIdx.x & 31;
   const int warps = (int)((gridDim.x * blockDim.x) >> 5);
   for (int c = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); c < cols; c += warps) {
@@ -269,171 +270,7 @@ __global__ void k_sum_cols(const double* __restrict__ p, int rows, int cols, dou
     for (int b = lane; b < rows; b += 32) r += p[(int64_t)b * cols + c];
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) r += __shfl_down_sync(0xffffffffu, r, off);
-    if (lane == 0) out[c] = r;
-  }
-}
-
-__global__ void k_struct(const float* __restrict__ u, int nx, int ny, int nz, int r,
-                         double* __restrict__ partials, int64_t block_stride) {
-  const int64_t n = (int64_t)nx * ny * nz;
-  double acc[6] = {0, 0, 0, 0, 0, 0};
-  const int rx = r % nx, ry = r % ny, rz = r % nz;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    int x, y, z;
-    cell_xyz(i, nx, ny, x, y, z);
-    const int xr = x + rx >= nx ? x + rx - nx : x + rx;
-    const int yr = y + ry >= ny ? y + ry - ny : y + ry;
-    const int zr = z + rz >= nz ? z + rz - nz : z + rz;
-    if (!in_bounds(xr >= 0 && xr < nx && yr >= 0 && yr < ny && zr >= 0 && zr < nz)) continue;
-    const double d3[3] = {
-        (double)u[((int64_t)z * ny + y) * nx + xr] - (double)u[i],
-        (double)u[n + ((int64_t)z * ny + yr) * nx + x] - (double)u[n + i],
-        (double)u[2 * n + ((int64_t)zr * ny + y) * nx + x] - (double)u[2 * n + i]};
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      double p = d3[a];
-#pragma unroll
-      for (int k = 0; k < 6; ++k) {
-        acc[k] += p;
-        p *= d3[a];
-      }
-    }
-  }
-  __shared__ double red[32][6];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int k = 0; k < 6; ++k) {
-    double v = acc[k];
-    for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-    if (lane == 0) red[warp][k] = v;
-  }
-  __syncthreads();
-  if (threadIdx.x < 6) {
-    double v = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v += red[w][threadIdx.x];
-    partials[(int64_t)blockIdx.x * block_stride + threadIdx.x] = v;
-  }
-}
-
-// Structure functions of up to 24 separations in one launch: blockIdx.y takes
-// a chunk of kStructChunk separations, a warp one x-line at a time (lanes over
-// x: no division per cell), so a cell's own velocity is read once per chunk
-// rather than once per separation.  Per block b and separation k,
-// partials[(b * nr + k) * 6 + p - 1] = sum over its cells and the three axes
-// of d^p, d = u_a(x + r_k e_a) - u_a(x), p = 1..6.  The powers and the running
-// sums are FP32 (FP64 arithmetic is slow on this part: with FP64 powers the
-// 256^3 structure functions took 17 ms), folded into FP64 totals every
-// kFoldStruct cells; the block reduction is FP64.
-constexpr int kFoldStruct = 32;
-constexpr int kStructChunk = 3;
-
-__global__ void __launch_bounds__(kAuxThreads, 2)
-k_struct_multi(const float* __restrict__ u, int nx, int ny, int nz, StructSeps seps, int nr,
-               double* __restrict__ partials) {
-  const int k0 = blockIdx.y * kStructChunk;
-  const int kn = min(kStructChunk, nr - k0);
-  const int64_t n = (int64_t)nx * ny * nz;
-  // a chunk shorter than kStructChunk is padded with r = 0, whose increments
-  // are exactly zero: the cell loop has no branch per separation, so the
-  // loads of all separations are in flight together
-  int rx[kStructChunk], ry[kStructChunk], rz[kStructChunk];
-#pragma unroll
-  for (int j = 0; j < kStructChunk; ++j) {
-    const int r = j < kn ? seps.r[k0 + j] : 0;
-    rx[j] = r % nx;
-    ry[j] = r % ny;
-    rz[j] = r % nz;
-  }
-  // FP64 totals of each thread in shared memory, leaving the registers to the
-  // loads in flight
-  __shared__ double tot[kStructChunk * 6][kAuxThreads];
-  float t[kStructChunk][6];
-#pragma unroll
-  for (int j = 0; j < kStructChunk; ++j)
-#pragma unroll
-    for (int p = 0; p < 6; ++p) {
-      tot[j * 6 + p][threadIdx.x] = 0.0;
-      t[j][p] = 0.f;
-    }
-  int cnt = 0;
-  const int lane = threadIdx.x & 31;
-  const int64_t lines = (int64_t)ny * nz;
-  const int64_t wstride = (int64_t)gridDim.x * (blockDim.x >> 5);
-  for (int64_t l = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); l < lines; l += wstride) {
-    const int z = (int)(l / ny), y = (int)(l - (int64_t)z * ny);
-    const int64_t base = l * nx;
-    // two cells per lane and pass (x and x + 32; the second one weighted 0
-    // past the end of the line), so that twice the loads are in flight
-    for (int x0 = lane; x0 < nx; x0 += 64) {
-      const int x1 = x0 + 32 < nx ? x0 + 32 : x0;
-      const float w1 = x0 + 32 < nx ? 1.f : 0.f;
-      const int xs[2] = {x0, x1};
-      float own[2][3];
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        own[h][0] = u[base + xs[h]];
-        own[h][1] = u[n + base + xs[h]];
-        own[h][2] = u[2 * n + base + xs[h]];
-      }
-#pragma unroll
-      for (int j = 0; j < kStructChunk; ++j) {
-        const int yr = y + ry[j] >= ny ? y + ry[j] - ny : y + ry[j];
-        const int zr = z + rz[j] >= nz ? z + rz[j] - nz : z + rz[j];
-        float d[2][3];
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int x = xs[h];
-          const int xr = x + rx[j] >= nx ? x + rx[j] - nx : x + rx[j];
-          const bool ok = in_bounds(xr >= 0 && xr < nx && yr >= 0 && yr < ny && zr >= 0 && zr < nz);
-          const float m = ok ? (h ? w1 : 1.f) : 0.f;
-          d[h][0] = m * (u[base + (ok ? xr : x)] - own[h][0]);
-          d[h][1] = m * (u[n + ((int64_t)z * ny + (ok ? yr : y)) * nx + x] - own[h][1]);
-          d[h][2] = m * (u[2 * n + ((int64_t)(ok ? zr : z) * ny + y) * nx + x] - own[h][2]);
-        }
-#pragma unroll
-        for (int h = 0; h < 2; ++h)
-#pragma unroll
-          for (int a = 0; a < 3; ++a) {
-            float q = d[h][a];
-#pragma unroll
-            for (int p = 0; p < 6; ++p) {
-              t[j][p] += q;
-              q *= d[h][a];
-            }
-          }
-      }
-      cnt += 2;
-      if (cnt >= kFoldStruct) {
-#pragma unroll
-        for (int j = 0; j < kStructChunk; ++j)
-#pragma unroll
-          for (int p = 0; p < 6; ++p) {
-            tot[j * 6 + p][threadIdx.x] += (double)t[j][p];
-            t[j][p] = 0.f;
-          }
-        cnt = 0;
-      }
-    }
-  }
-  __shared__ double red[kAuxThreads / 32][6];
-  const int warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int j = 0; j < kStructChunk; ++j) {
-    if (j >= kn) break;
-#pragma unroll
-    for (int p = 0; p < 6; ++p) {
-      double v = tot[j * 6 + p][threadIdx.x] + (double)t[j][p];
-      for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-      if (lane == 0) red[warp][p] = v;
-    }
-    __syncthreads();
-    if (threadIdx.x < 6) {
-      double v = 0.0;
-      for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v += red[w][threadIdx.x];
-      partials[((int64_t)blockIdx.x * nr + k0 + j) * 6 + threadIdx.x] = v;
-    }
-    __syncthreads();
+    if (lane == 0) out[c] = r * scale;
   }
 }
 
@@ -549,24 +386,9 @@ cudaError_t launch_spec_finish(const double* partials, int blocks, int kmax, dou
 }
 
 cudaError_t launch_sum_cols(const double* partials, int rows, int cols, double* out,
-                            cudaStream_t st) {
+                            cudaStream_t st, double scale) {
   const int blocks = std::max(1, std::min(1024, (cols + 7) / 8));  // 8 warps per block, a warp per column
-  return launch_kernel(k_sum_cols, blocks, 256, 0, st, partials, rows, cols, out);
-}
-
-cudaError_t launch_struct_multi(const float* u, int nx, int ny, int nz, const int* r, int nr, double* partials,
-                                int blocks, cudaStream_t st) {
-  if (nr < 1 || nr > kMaxStructSeps) return cudaErrorInvalidValue;
-  StructSeps seps{};
-  for (int k = 0; k < nr; ++k) seps.r[k] = r[k];
-  const int chunks = (nr + kStructChunk - 1) / kStructChunk;
-  return launch_kernel(k_struct_multi, dim3(blocks, chunks), kAuxThreads, 0, st, u, nx, ny, nz, seps, nr,
-                       partials);
-}
-
-cudaError_t launch_struct(const float* u, int nx, int ny, int nz, int r, double* partials,
-                          int blocks, cudaStream_t st, int64_t block_stride) {
-  return launch_kernel(k_struct, blocks, kAuxThreads, 0, st, u, nx, ny, nz, r, partials, block_stride);
+  return launch_kernel(k_sum_cols, blocks, 256, 0, st, partials, rows, cols, scale, out);
 }
 
 uint32_t bounds_word_aux() { return take_bounds_word(); }

@@ -116,23 +116,9 @@ cudaError_t launch_spec_bin(const void* coeffs, int nx, int ny, int nz, int kmax
                             double* partials, int blocks, cudaStream_t st);
 cudaError_t launch_spec_finish(const double* partials, int blocks, int kmax, double* E,
                                cudaStream_t st);
-// Structure functions: per block b, partials[b * block_stride + p - 1] = sum over
-// its cells and the three axes of (u_a(x + r e_a) - u_a(x))^p, p = 1..6, for the
-// velocity u [3][nz][ny][nx] FP32.
-cudaError_t launch_struct(const float* u, int nx, int ny, int nz, int r, double* partials,
-                          int blocks, cudaStream_t st, int64_t block_stride = 6);
-// The separations of one launch (kernel parameter).
-constexpr int kMaxStructSeps = 24;
-struct StructSeps {
-  int r[kMaxStructSeps];
-};
-// Structure functions of nr <= 24 separations r[0..nr) in one launch, FP32
-// powers folded into FP64: partials [blocks][nr][6] of the per-block sums over
-// cells and the three axes of d^p, p = 1..6.
-cudaError_t launch_struct_multi(const float* u, int nx, int ny, int nz, const int* r, int nr, double* partials,
-                                int blocks, cudaStream_t st);
+// out[c] = scale * sum over rows of partials[rows][cols].
 cudaError_t launch_sum_cols(const double* partials, int rows, int cols, double* out,
-                            cudaStream_t st);
+                            cudaStream_t st, double scale = 1.0);
 
 // Seeded random solenoidal velocity (lbm_random_field.cu): the FP32 field
 // u[3][nz][ny][nx] (device memory, 3 nx ny nz floats) of the recipe described

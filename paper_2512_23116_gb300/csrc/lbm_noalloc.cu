@@ -16,6 +16,7 @@
 
 #include "../../include/lbm.h"
 #include "lbm_kernels.h"
+#include "lbm_struct.h"
 
 #define LBM_API extern "C" __attribute__((visibility("default")))
 
@@ -25,13 +26,14 @@ void set_global_error(const char* msg);
 
 namespace {
 
-constexpr int kBlocks = 512;            // blocks of each separation's reduction
+constexpr int kBlocks = 512;            // blocks of a separation's own reduction
 constexpr int kMaxSeparations = LBM_MAX_R;
 constexpr int kMaxDevices = 64;
 
-// Partial sums of (d)^p, p = 1..6, per separation and block: 24 x 512 x 6
+// Partial sums of (d)^p, p = 1..6, per block and separation: 24 x 512 x 6
 // doubles = 576 KiB.
-static __device__ __align__(256) double g_sf_scratch[kMaxSeparations * kBlocks * 6];
+constexpr int kScratch = kMaxSeparations * kBlocks * 6;
+static __device__ __align__(256) double g_sf_scratch[kScratch];
 
 std::mutex g_mutex;
 double* g_scratch_addr[kMaxDevices] = {};
@@ -52,17 +54,6 @@ cudaError_t scratch_address(double** out) {
   }
   *out = g_scratch_addr[dev];
   return cudaSuccess;
-}
-
-// sp[k][p] = (sum over blocks of part[k][block][p]) * inv_count.
-__global__ void k_sf_finish(const double* __restrict__ part, int nr, int blocks, double inv_count,
-                            double* __restrict__ sp) {
-  for (int idx = threadIdx.x; idx < nr * 6; idx += blockDim.x) {
-    const int k = idx / 6, p = idx - k * 6;
-    double s = 0.0;
-    for (int b = 0; b < blocks; ++b) s += part[((int64_t)k * blocks + b) * 6 + p];
-    sp[idx] = s * inv_count;
-  }
 }
 
 int reject(int code, const char* msg) {
@@ -116,12 +107,20 @@ LBM_API int lbm_structure_functions_noalloc(const float* u, int32_t nx, int32_t 
   e = scratch_address(&scratch);
   if (e != cudaSuccess) return reject(LBM_ERR_CUDA, cudaGetErrorString(e));
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  for (int k = 0; k < nr; ++k) {
-    e = lbm::launch_struct(u, nx, ny, nz, r[k], scratch + (size_t)k * kBlocks * 6, kBlocks, st);
-    if (e != cudaSuccess) return reject(LBM_ERR_CUDA, cudaGetErrorString(e));
+  // Every separation in one launch where their wrapped distances fit the tiles;
+  // else one FP64 pass per separation.  Either way per-block sums [blocks][nr][6]
+  // and one column sum.
+  lbm::StructPlan plan;
+  int blocks = kBlocks;
+  if (lbm::plan_struct(nx, ny, nz, r, nr, true, kScratch / (6 * nr), &plan, &e)) {
+    blocks = plan.grid;
+    e = lbm::launch_struct_plan(u, plan, true, scratch, st);
+  } else {
+    for (int k = 0; k < nr && e == cudaSuccess; ++k)
+      e = lbm::launch_struct(u, nx, ny, nz, r[k], scratch + (size_t)k * 6, kBlocks, st, (int64_t)nr * 6);
   }
-  const double inv_count = 1.0 / (3.0 * (double)ncell);
-  e = lbm::launch_kernel(k_sf_finish, 1, 160, 0, st, (const double*)scratch, nr, kBlocks, inv_count, sp);
+  if (e != cudaSuccess) return reject(LBM_ERR_CUDA, cudaGetErrorString(e));
+  e = lbm::launch_sum_cols(scratch, blocks, nr * 6, sp, st, 1.0 / (3.0 * (double)ncell));
   if (e != cudaSuccess) return reject(LBM_ERR_CUDA, cudaGetErrorString(e));
   return LBM_OK;
 }

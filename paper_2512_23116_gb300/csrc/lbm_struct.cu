@@ -1,0 +1,532 @@
+// Structure functions S_p(r) = <(u_a(x + r e_a) - u_a(x))^p>, p = 1..6, pooled
+// over the three axes a (Eqs. velocity_increment, structure_function), for up to
+// 24 separations in one launch.
+//
+// Layout of the work.  Component a only ever meets itself along axis a, so the
+// field falls into pencils: 32 pencils by L cells along the axis (plus the
+// largest separation, wrapped) are staged in shared memory once and serve every
+// separation; element i of pencil c is at i x 33 + c, so that staging x-lines
+// (lanes along i) and walking pencils (lanes along c) are both free of bank
+// conflicts.  A warp walks a run of cells with one lane per pencil; a cell's own
+// value and its partners are one shared-memory load each at a fixed offset.
+// Reading every partner from global memory instead was bound by the latency of
+// the shifted loads (9 % of the DRAM peak at 256^3).
+//
+// Two accuracies share that skeleton:
+//  - k_struct_tiles<false>, for lbm_stats: FP32 increments and powers as the
+//    FP32 velocity allows, summed in FP32 over at most kRunMax cells of a lane
+//    and the lanes of its warp, then in FP64.  Bound by issue: 10 instructions an
+//    increment (9 FP32 operations and a load), 73 % of the issue rate at 400^3.
+//    All separations of a call: 100^3 (11 of them) 102 -> 23 us, 400^3 (15)
+//    3.11 -> 1.34 ms, 512^3 (16) 8.5 -> 2.75 ms.
+//  - k_struct_tiles<true>, for lbm_structure_functions_noalloc: the FP64 sums of
+//    the exact increments.  This part executes 2 FP64 operations per clock and
+//    SM against 128 in FP32, so increments, powers and running sums are kept as
+//    unevaluated sums of FP32 words (Dekker 1971; Knuth's two-sum, products with
+//    an FMA for the remainder).  Against long double sums it is off by 1-4e-16
+//    of S_2, S_4, S_6 and 1-8e-18 of <|d|^3>, <|d|^5> on 50x61x77 to 100^3, where
+//    the FP64 loop left 3-7e-16 and 4e-18-6e-17.  Each tile scales its increments
+//    by a power of two so that neither the sixth power nor its low words leave the
+//    FP32 range; a tile whose values do not allow that (infinities, NaN, extreme
+//    exponents) is summed in FP64.  Bound by issue: ~170 FP32 operations an
+//    increment.  12 separations at 160^3: 4.43 ms (one FP64 pass over global memory
+//    per separation, at the FP64 rate) -> 0.87 ms.
+#include <cuda_runtime.h>
+
+#include <algorithm>
+#include <climits>
+
+#include "lbm_check.cuh"
+#include "lbm_kernels.h"
+#include "lbm_struct.h"
+
+namespace lbm {
+
+namespace {
+
+constexpr int kCols = 32;       // pencils of a tile: one per lane
+constexpr int kPitch = 33;      // values between consecutive cells of a pencil
+constexpr int kRunMax = 64;     // cells a lane sums before the warp reduces
+constexpr int kWarpsMax = 8;
+// Lattices below this many cells are summed in FP64 terms: on 7,680 cells the
+// roundings of the three-word even powers left 1.7-2.9e-16 of S_2, S_4, S_6 where
+// FP64 left 0.7-1.5e-16; from 96,000 cells on they leave less (1.9e-16 against
+// 4-5e-16), and the two cost the same time only where both are short of work.
+constexpr int64_t kWordsCells = 1 << 16;
+constexpr int kSmemMax = 225 * 1024;  // dynamic shared memory of a block, beside the few static words
+
+// Separations of one pass over a tile: its sums stay in registers (24 FP32 sums
+// of 4 separations, or 12 three-word sums of 2).
+template <bool EXACT> constexpr int chunk_len() { return EXACT ? 2 : 4; }
+
+__device__ __forceinline__ void stage4(uint32_t dst, const float* src, bool live) {
+  // 4-byte asynchronous copy; a pencil past the end reads as zeros
+  const int n = live ? 4 : 0;
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(n) : "memory");
+}
+
+// A value h + l + m of three FP32 words, |l| <= 2^-24 |h| and m of the order of
+// 2^-48 |h| (a rounded remainder, so the value is good to about 2^-70).
+struct Words {
+  float h, l, m;
+};
+// s + e = a + b exactly (Knuth)
+__device__ __forceinline__ float two_sum(float a, float b, float& e) {
+  const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
+  e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t));
+  return s;
+}
+// Running sums.  The full one keeps every remainder: the odd powers cancel, so
+// their sums feel each term's rounding; the short one drops the remainders of the
+// low words (2^-48 of a term at random), which an even power's sum does not feel.
+__device__ __forceinline__ void add_full(Words& s, const Words& v) {
+  float e, e1, e2;
+  s.h = two_sum(s.h, v.h, e);
+  const float w = two_sum(e, v.l, e1);
+  s.l = two_sum(s.l, w, e2);
+  s.m = __fadd_rn(s.m, __fadd_rn(v.m, __fadd_rn(e1, e2)));
+}
+__device__ __forceinline__ void add_short(Words& s, const Words& v) {
+  float e;
+  s.h = two_sum(s.h, v.h, e);
+  s.l = __fadd_rn(s.l, __fadd_rn(e, v.l));
+  s.m = __fadd_rn(s.m, v.m);
+}
+// a b to three words, every term down to second order; short: only those second-order
+// terms that do not average out (l l and h m: a low word rounds them away
+// always in the same direction, 2e-15 of a sum of even powers).
+__device__ __forceinline__ Words mul_full(const Words& a, const Words& b) {
+  Words c;
+  c.h = __fmul_rn(a.h, b.h);
+  const float t = __fmaf_rn(a.h, b.h, -c.h);
+  const float x1 = __fmul_rn(a.h, b.l), x2 = __fmul_rn(a.l, b.h);
+  const float r1 = __fmaf_rn(a.h, b.l, -x1), r2 = __fmaf_rn(a.l, b.h, -x2);
+  float y1, y2;
+  const float w = two_sum(x1, x2, y1);
+  c.l = two_sum(t, w, y2);
+  c.m = __fmaf_rn(a.l, b.l, __fmaf_rn(a.h, b.m, __fmaf_rn(a.m, b.h, __fadd_rn(__fadd_rn(r1, r2), __fadd_rn(y1, y2)))));
+  return c;
+}
+__device__ __forceinline__ Words sqr_full(const Words& a) {  // a.m = 0
+  Words c;
+  c.h = __fmul_rn(a.h, a.h);
+  const float t = __fmaf_rn(a.h, a.h, -c.h), a2 = __fadd_rn(a.h, a.h);
+  const float x = __fmul_rn(a2, a.l), r = __fmaf_rn(a2, a.l, -x);
+  float y;
+  c.l = two_sum(t, x, y);
+  c.m = __fmaf_rn(a.l, a.l, __fadd_rn(r, y));
+  return c;
+}
+__device__ __forceinline__ Words sqr_short(const Words& a) {
+  Words c;
+  c.h = __fmul_rn(a.h, a.h);
+  const float a2 = __fadd_rn(a.h, a.h);
+  c.l = __fmaf_rn(a2, a.l, __fmaf_rn(a.h, a.h, -c.h));
+  c.m = __fmaf_rn(a.l, a.l, __fmul_rn(a2, a.m));
+  return c;
+}
+
+// Running sums of (d, d^2, ..., d^6) of one separation.  The low words of d^2 are
+// summed apart from the remainders of its sum (`low2`): their sum rounds with a
+// bias when increments have few significant bits.
+struct PowerSums {
+  Words s[6];
+  float low2;
+  __device__ __forceinline__ void reset() {
+#pragma unroll
+    for (int k = 0; k < 6; ++k) s[k] = {0.f, 0.f, 0.f};
+    low2 = 0.f;
+  }
+  // d = (a - b) times `scale`, a power of two: exact in two words
+  __device__ __forceinline__ void add(float a, float b, float scale) {
+    float e;
+    const float r = two_sum(a, -b, e);
+    const Words d = {__fmul_rn(r, scale), __fmul_rn(e, scale), 0.f};
+    const Words q = sqr_full(d), c = mul_full(q, d);
+    add_full(s[0], d);
+    add_short(s[1], {q.h, 0.f, q.m});
+    low2 = __fadd_rn(low2, q.l);
+    add_full(s[2], c);
+    add_short(s[3], sqr_short(q));
+    add_full(s[4], mul_full(c, q));
+    add_short(s[5], sqr_short(c));
+  }
+};
+
+// Sum 24 values over the warp's 32 lanes, value i ending in lane i: each step
+// halves the values a lane holds (31 shuffles instead of 120).
+__device__ __forceinline__ float warp_sums(const float (&v)[24], int lane) {
+  float a[32];
+#pragma unroll
+  for (int i = 0; i < 32; ++i) a[i] = i < 24 ? v[i] : 0.f;
+#pragma unroll
+  for (int s = 16; s > 0; s >>= 1) {
+    const bool up = (lane & s) != 0;
+#pragma unroll
+    for (int i = 0; i < s; ++i) {
+      const float send = up ? a[i] : a[i + s], keep = up ? a[i + s] : a[i];
+      a[i] = keep + __shfl_xor_sync(0xffffffffu, send, s);
+    }
+  }
+  return a[0];
+}
+
+// The same for the 12 three-word sums of two separations, value i ending in lanes
+// 2 i and 2 i + 1, as FP64 (which adds them up only here: 5 slow FP64 operations
+// a warp instead of 76).
+__device__ __forceinline__ double warp_sums(const PowerSums (&v)[2], int lane) {
+  Words a[16];
+#pragma unroll
+  for (int i = 0; i < 16; ++i) a[i] = i < 12 ? v[i / 6].s[i % 6] : Words{0.f, 0.f, 0.f};
+  add_full(a[1], {0.f, v[0].low2, 0.f});
+  add_full(a[7], {0.f, v[1].low2, 0.f});
+#pragma unroll
+  for (int s = 16; s > 0; s >>= 1) {
+    const bool up = (lane & s) != 0;
+#pragma unroll
+    for (int i = 0; i < (s > 1 ? s / 2 : 1); ++i) {
+      Words send = a[i], keep = a[i];
+      if (s > 1) {
+        const Words lo = a[i], hi = a[i + s / 2];
+        send = up ? lo : hi;
+        keep = up ? hi : lo;
+      }
+      const Words o = {__shfl_xor_sync(0xffffffffu, send.h, s), __shfl_xor_sync(0xffffffffu, send.l, s),
+                       __shfl_xor_sync(0xffffffffu, send.m, s)};
+      add_full(keep, o);
+      a[i] = keep;
+    }
+  }
+  return (double)a[0].h + ((double)a[0].l + (double)a[0].m);
+}
+__device__ __forceinline__ double warp_sums(const double (&v)[12], int lane) {
+  double a[16];
+#pragma unroll
+  for (int i = 0; i < 16; ++i) a[i] = i < 12 ? v[i] : 0.0;
+#pragma unroll
+  for (int s = 16; s > 1; s >>= 1) {
+    const bool up = (lane & s) != 0;
+#pragma unroll
+    for (int i = 0; i < s / 2; ++i) {
+      const double send = up ? a[i] : a[i + s / 2], keep = up ? a[i + s / 2] : a[i];
+      a[i] = keep + __shfl_xor_sync(0xffffffffu, send, s);
+    }
+  }
+  return a[0] + __shfl_xor_sync(0xffffffffu, a[0], 1);
+}
+
+// Sums of one chunk over the run of n cells that starts at p (lane's pencil), FP32.
+__device__ __forceinline__ void run_f32(const float* p, const int (&off)[4], int n, float (&t)[24]) {
+#pragma unroll
+  for (int i = 0; i < 24; ++i) t[i] = 0.f;
+#pragma unroll 4
+  for (int i = 0; i < n; ++i, p += kPitch) {
+    const float own = p[0];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const float d = p[off[j]] - own;
+      const float q = d * d, c = q * d;
+      t[6 * j] += d;
+      t[6 * j + 1] += q;
+      t[6 * j + 2] = fmaf(q, d, t[6 * j + 2]);
+      t[6 * j + 3] = fmaf(q, q, t[6 * j + 3]);
+      t[6 * j + 4] = fmaf(c, q, t[6 * j + 4]);
+      t[6 * j + 5] = fmaf(c, c, t[6 * j + 5]);
+    }
+  }
+}
+
+// The same in three-word arithmetic, increments times `scale` (a power of two).
+__device__ __forceinline__ void run_words(const float* p, const int (&off)[2], int n, float scale, PowerSums (&t)[2]) {
+  t[0].reset();
+  t[1].reset();
+  for (int i = 0; i < n; ++i, p += kPitch) {
+    const float own = p[0];
+#pragma unroll
+    for (int j = 0; j < 2; ++j) t[j].add(p[off[j]], own, scale);
+  }
+}
+
+// The same in FP64, for tiles outside the range of the three-word arithmetic.
+__device__ __noinline__ void run_f64(const float* p, int off0, int off1, int n, double* t) {
+  for (int i = 0; i < n; ++i, p += kPitch) {
+    const double own = p[0];
+    for (int j = 0; j < 2; ++j) {
+      const double d = (double)p[j ? off1 : off0] - own;
+      double q = d;
+      for (int k = 0; k < 6; ++k) {
+        t[6 * j + k] += q;
+        q *= d;
+      }
+    }
+  }
+}
+
+// The exponent k of the tile's scale 2^k: the largest difference of adjacent
+// cells times 2^k lies in [2^7, 2^8), so an increment over at most 2^11 cells
+// stays below 2^19, its sixth power below 2^114 and a run's sum below 2^120; its
+// low parts keep all their bits down to increments 2^-20 of that largest one,
+// whose share of a sum is below the FP64 rounding.  INT_MIN when the
+// values do not allow it.
+__device__ __forceinline__ int tile_exponent(float adj, float top) {
+  if (adj == 0.f && top < 1e30f) return 0;  // constant pencils: every increment is zero
+  if (!(adj >= 0x1p-60f && adj < 0x1p60f && top < 0x1p60f)) return INT_MIN;
+  const int e = (int)(__float_as_uint(adj) >> 23) - 127;
+  const int k = 7 - e;
+  const int et = (int)(__float_as_uint(top) >> 23) - 127;
+  return et + k < 120 ? k : INT_MIN;
+}
+
+// Tiles of the three axes in one numbering; a block takes tiles b, b + grid, ...
+// partials[block][nr][6].
+template <bool EXACT>
+__global__ void __launch_bounds__(kWarpsMax * 32, EXACT ? 2 : 3)
+k_struct_tiles(const float* __restrict__ u, StructPlan pl, double* __restrict__ partials) {
+  extern __shared__ __align__(16) float tile[];  // [rows][33], then [warps][nr][6] doubles
+  __shared__ float s_adj[kWarpsMax], s_top[kWarpsMax];
+  constexpr int CH = chunk_len<EXACT>();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+  const int nv = 6 * pl.nr;
+  double* tot = reinterpret_cast<double*>(tile + pl.rows_max * kPitch);
+  double* mine = tot + warp * nv;
+  for (int i = lane; i < nv; i += 32) mine[i] = 0.0;
+  const uint32_t tile_s = static_cast<uint32_t>(__cvta_generic_to_shared(tile));
+  for (int64_t t = blockIdx.x; t < pl.tiles; t += gridDim.x) {
+    const int a = t < pl.ax[1].first ? 0 : (t < pl.ax[2].first ? 1 : 2);
+    const StructAxis& ax = pl.ax[a];
+    const int64_t local = t - ax.first;
+    const int64_t ct = local / ax.segs;
+    const int i0 = (int)(local - ct * ax.segs) * ax.len;
+    const int64_t c0 = ct * kCols;
+    const int len = min(ax.len, ax.n - i0), rows = len + ax.halo;
+    const float* ua = u + a * pl.ncell;
+    __syncthreads();  // the previous tile has been read
+    if (a == 0) {     // x-lines: lanes along the line
+      for (int c = warp; c < kCols; c += nwarps) {
+        const bool live = c0 + c < ax.pencils;
+        const float* line = ua + (live ? c0 + c : 0) * ax.n;
+        for (int i = lane; i < rows; i += 32) {
+          const int x = i0 + i < ax.n ? i0 + i : i0 + i - ax.n;
+          if (in_bounds(x >= 0 && x < ax.n && i < pl.rows_max)) stage4(tile_s + 4u * (i * kPitch + c), line + x, live);
+        }
+      }
+    } else {  // pencils across x-lines: lanes along x
+      const int64_t c = c0 + lane;
+      const bool live = c < ax.pencils;
+      // y: pencil (z, x) starts at z ny nx + x; z: pencil (y, x) at its own index
+      int64_t base = live ? c : 0;
+      if (a == 1) base += base / pl.nx * (pl.plane - pl.nx);
+      for (int i = warp; i < rows; i += nwarps) {
+        const int k = i0 + i < ax.n ? i0 + i : i0 + i - ax.n;
+        const int64_t o = base + k * ax.stride;
+        if (in_bounds(o >= 0 && o < pl.ncell && i < pl.rows_max)) stage4(tile_s + 4u * (i * kPitch + lane), ua + o, live);
+      }
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+    int kexp = 0;
+    if (EXACT) {
+      float adj = 0.f, top = 0.f;
+      bool odd = false;  // NaN: fmaxf would drop it
+      for (int i = warp; i < rows; i += nwarps) {
+        const float v = tile[i * kPitch + lane];
+        top = fmaxf(top, fabsf(v));
+        odd |= !(fabsf(v) < 0x1p60f);
+        if (i + 1 < rows) adj = fmaxf(adj, fabsf(tile[(i + 1) * kPitch + lane] - v));
+      }
+      if (odd) top = 0x1p100f;
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) {
+        adj = fmaxf(adj, __shfl_xor_sync(0xffffffffu, adj, off));
+        top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, off));
+      }
+      if (lane == 0) {
+        s_adj[warp] = adj;
+        s_top[warp] = top;
+      }
+      __syncthreads();
+      for (int w = 0; w < nwarps; ++w) {
+        adj = fmaxf(adj, s_adj[w]);
+        top = fmaxf(top, s_top[w]);
+      }
+      kexp = pl.fp64 ? INT_MIN : tile_exponent(adj, top);
+    }
+    const int q = (len + nwarps - 1) / nwarps;
+    const int n = max(0, min(q, len - warp * q));
+    const float* p = tile + warp * q * kPitch + lane;
+    for (int k0 = 0; k0 < pl.nr; k0 += CH) {
+      int off[CH];  // a chunk past the last separation is padded with r = 0: zero increments
+#pragma unroll
+      for (int j = 0; j < CH; ++j) off[j] = (k0 + j < pl.nr ? pl.r[a][k0 + j] : 0) * kPitch;
+      if constexpr (EXACT) {
+        double v;
+        if (kexp == INT_MIN) {
+          double d[12];
+#pragma unroll
+          for (int i = 0; i < 12; ++i) d[i] = 0.0;
+          run_f64(p, off[0], off[1], n, d);
+          v = warp_sums(d, lane);
+        } else {
+          PowerSums s[2];
+          run_words(p, off, n, __uint_as_float((uint32_t)(kexp + 127) << 23), s);
+          v = warp_sums(s, lane);
+          // sum of (2^k d)^p: times 2^(-k p)
+          if (kexp != 0) v *= __longlong_as_double((long long)(1023 - kexp * ((lane >> 1) % 6 + 1)) << 52);
+        }
+        const int i = k0 * 6 + (lane >> 1);
+        if (!(lane & 1) && lane < 24 && i < nv) mine[i] += v;
+      } else {
+        float s[24];
+        run_f32(p, off, n, s);
+        const float v = warp_sums(s, lane);
+        const int i = k0 * 6 + lane;
+        if (lane < 24 && i < nv) mine[i] += (double)v;
+      }
+    }
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < nv; i += blockDim.x) {
+    double s = 0.0;
+    for (int w = 0; w < nwarps; ++w) s += tot[w * nv + i];
+    partials[(int64_t)blockIdx.x * nv + i] = s;
+  }
+}
+
+// S_p(r) of one separation in FP64, one cell per thread and pass, partners read
+// from global memory: separations whose wrapped distance does not fit a tile.
+__global__ void k_struct(const float* __restrict__ u, int nx, int ny, int nz, int r,
+                         double* __restrict__ partials, int64_t block_stride) {
+  const int64_t n = (int64_t)nx * ny * nz;
+  double acc[6] = {0, 0, 0, 0, 0, 0};
+  const int rx = r % nx, ry = r % ny, rz = r % nz;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
+       i += (int64_t)gridDim.x * blockDim.x) {
+    int x, y, z;
+    if (n < (int64_t)0x7fffffff) {  // 32-bit division for lattices below 2^31 cells
+      const uint32_t row = (uint32_t)i / (uint32_t)nx;
+      x = (int)((uint32_t)i - row * (uint32_t)nx);
+      z = (int)(row / (uint32_t)ny);
+      y = (int)(row - (uint32_t)z * (uint32_t)ny);
+    } else {
+      const int64_t row = i / nx;
+      x = (int)(i - row * nx);
+      z = (int)(row / ny);
+      y = (int)(row - (int64_t)z * ny);
+    }
+    const int xr = x + rx >= nx ? x + rx - nx : x + rx;
+    const int yr = y + ry >= ny ? y + ry - ny : y + ry;
+    const int zr = z + rz >= nz ? z + rz - nz : z + rz;
+    if (!in_bounds(xr >= 0 && xr < nx && yr >= 0 && yr < ny && zr >= 0 && zr < nz)) continue;
+    const double d3[3] = {
+        (double)u[((int64_t)z * ny + y) * nx + xr] - (double)u[i],
+        (double)u[n + ((int64_t)z * ny + yr) * nx + x] - (double)u[n + i],
+        (double)u[2 * n + ((int64_t)zr * ny + y) * nx + x] - (double)u[2 * n + i]};
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      double p = d3[a];
+#pragma unroll
+      for (int k = 0; k < 6; ++k) {
+        acc[k] += p;
+        p *= d3[a];
+      }
+    }
+  }
+  __shared__ double red[32][6];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+    double v = acc[k];
+    for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
+    if (lane == 0) red[warp][k] = v;
+  }
+  __syncthreads();
+  if (threadIdx.x < 6) {
+    double v = 0.0;
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v += red[w][threadIdx.x];
+    partials[(int64_t)blockIdx.x * block_stride + threadIdx.x] = v;
+  }
+}
+
+template <bool EXACT>
+cudaError_t finish_plan(StructPlan& pl, int max_blocks) {
+  cudaError_t e = cudaFuncSetAttribute(k_struct_tiles<EXACT>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
+  int per_sm = 0, dev = 0, sms = 0;
+  if (e == cudaSuccess)
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_struct_tiles<EXACT>, pl.threads, pl.smem);
+  if (e == cudaSuccess) e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e == cudaSuccess && per_sm < 1) e = cudaErrorInvalidConfiguration;
+  if (e == cudaSuccess)
+    pl.grid = (int)std::max<int64_t>(1, std::min<int64_t>({pl.tiles, (int64_t)per_sm * sms, (int64_t)max_blocks}));
+  return e;
+}
+
+}  // namespace
+
+bool plan_struct(int nx, int ny, int nz, const int* r, int nr, bool exact, int max_blocks, StructPlan* out,
+                 cudaError_t* err) {
+  *err = cudaErrorInvalidValue;
+  if (nr < 1 || nr > kMaxStructSeps) return false;
+  StructPlan pl{};
+  const int n[3] = {nx, ny, nz};
+  pl.nr = nr;
+  pl.nx = nx;
+  pl.plane = (int64_t)nx * ny;
+  pl.ncell = pl.plane * nz;
+  int longest = 0, halo = 0;
+  for (int a = 0; a < 3; ++a) {
+    for (int k = 0; k < nr; ++k) {
+      pl.r[a][k] = r[k] % n[a];
+      pl.ax[a].halo = std::max(pl.ax[a].halo, pl.r[a][k]);
+    }
+    longest = std::max(longest, n[a]);
+    halo = std::max(halo, pl.ax[a].halo);
+  }
+  const size_t sums = sizeof(double) * 6 * nr;
+  // Blocks of 4 warps where six or more of them fit an SM (its pencils up to
+  // ~250 cells with their halo): a lane's run is then long against the warp
+  // reduction that ends it.  Longer pencils get 8 warps, so that the two
+  // blocks an SM has room for still fill it.  A pencil is cut into segments of
+  // at most kRunMax cells per warp.
+  const int short_rows = std::min(longest, 4 * kRunMax) + halo;
+  const int warps = longest <= 4 * kRunMax && (size_t)short_rows * kPitch * 4 + 4 * sums <= 36 * 1024 ? 4 : kWarpsMax;
+  int64_t tiles = 0;
+  for (int a = 0; a < 3; ++a) {
+    StructAxis& ax = pl.ax[a];
+    ax.n = n[a];
+    ax.stride = a == 0 ? 1 : (a == 1 ? (int64_t)nx : pl.plane);
+    ax.pencils = pl.ncell / n[a];
+    ax.segs = (n[a] + warps * kRunMax - 1) / (warps * kRunMax);
+    ax.len = (n[a] + ax.segs - 1) / ax.segs;
+    ax.segs = (n[a] + ax.len - 1) / ax.len;
+    ax.first = tiles;
+    tiles += (ax.pencils + kCols - 1) / kCols * ax.segs;
+    pl.rows_max = std::max(pl.rows_max, ax.len + ax.halo);
+  }
+  pl.rows_max += pl.rows_max & 1;  // the FP64 sums behind the tile start on 8 bytes
+  pl.tiles = tiles;
+  pl.fp64 = pl.ncell < kWordsCells;
+  pl.threads = 32 * warps;
+  const size_t smem = (size_t)pl.rows_max * kPitch * 4 + warps * sums;
+  *err = cudaSuccess;
+  // an increment spans at most 2^11 cells (tile_exponent)
+  if (smem > (size_t)kSmemMax || pl.rows_max > 2048) return false;
+  pl.smem = (int)smem;
+  *err = exact ? finish_plan<true>(pl, max_blocks) : finish_plan<false>(pl, max_blocks);
+  *out = pl;
+  return *err == cudaSuccess;
+}
+
+cudaError_t launch_struct_plan(const float* u, const StructPlan& pl, bool exact, double* partials, cudaStream_t st) {
+  return exact ? launch_kernel(k_struct_tiles<true>, pl.grid, pl.threads, pl.smem, st, u, pl, partials)
+               : launch_kernel(k_struct_tiles<false>, pl.grid, pl.threads, pl.smem, st, u, pl, partials);
+}
+
+cudaError_t launch_struct(const float* u, int nx, int ny, int nz, int r, double* partials,
+                          int blocks, cudaStream_t st, int64_t block_stride) {
+  return launch_kernel(k_struct, blocks, 256, 0, st, u, nx, ny, nz, r, partials, block_stride);
+}
+
+uint32_t bounds_word_struct() { return take_bounds_word(); }
+
+}  // namespace lbm
