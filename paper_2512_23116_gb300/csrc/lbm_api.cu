@@ -22,6 +22,7 @@
 #include "lbm_check.cuh"
 #include "lbm_internal.h"
 #include "lbm_kernels.h"
+#include "lbm_spectrum.h"
 #include "lbm_struct.h"
 
 #define LBM_API extern "C" __attribute__((visibility("default")))
@@ -33,6 +34,7 @@ using namespace lbm;
 constexpr int kRingCap = 1024;
 constexpr int kMinHistWindow = 256;  // fewer histogram bins than this in shared memory: all global
 constexpr int64_t kChunkCells = 4 << 20;
+constexpr size_t kFftBatchBytes = 192 << 20;  // three half spectra (256^3) transformed together
 constexpr double kPi = 3.14159265358979323846;
 
 thread_local std::string g_create_error;
@@ -55,8 +57,13 @@ struct Inst {
   float* plane = nullptr;   // largest plane
   uint32_t* hist = nullptr; // [hist_bins + 1]
   bool has_plan = false;
-  cufftHandle plan = 0;
-  void* fft_out = nullptr;
+  cufftHandle plan = 0;     // extents the framework's own transform does not take
+  FftPlan fft;              // its plan for fft_kmax shells (when fft_own)
+  int fft_kmax = -1;
+  bool fft_own = false;
+  float2* fft_tw = nullptr; // its twiddle tables
+  void* fft_out = nullptr;  // half spectra
+  size_t fft_bytes = 0;
   uint64_t rec_read = 0;
   // what the diagnostic buffers hold: u of state version u_version; the
   // spectrum (shells 0..spec_kmax) of state version spec_version
@@ -439,7 +446,7 @@ int check_err(lbm_t h) {
   CK(h, cudaStreamSynchronize(h->stream));
   if (kBoundsCheck) {
     const uint32_t b = bounds_word_tma() | bounds_word_direct() | bounds_word_aux() | bounds_word_random() |
-                       bounds_word_struct();
+                       bounds_word_struct() | bounds_word_spectrum();
     if (b) return fail(h, LBM_ERR_CUDA, "device bounds check failed (checked build; word %u)", b);
   }
   if (e) {
@@ -606,27 +613,68 @@ int spectrum_device(lbm_t h, int i, int kmax, double* host_E) {
     std::copy(I.spec_E.begin(), I.spec_E.begin() + kmax + 1, host_E);
     return LBM_OK;
   }
-  if (!I.has_plan) {
+  if (I.fft_kmax != kmax) {
+    cudaError_t pe;
+    I.fft_own = plan_fft(p.nx, p.ny, p.nz, kmax, &I.fft, &pe);
+    CK(h, pe);
+    I.fft_kmax = kmax;
+  }
+  // Own transform: all three components in one launch per pass while their half
+  // spectra together stay small (the launches are what small lattices pay
+  // for), else one after the other through one buffer.
+  const size_t one = I.fft_own ? sizeof(float2) * (size_t)I.fft.half
+                               : sizeof(float2) * (size_t)p.nz * p.ny * (p.nx / 2 + 1);
+  const int comps = I.fft_own && 3 * one <= kFftBatchBytes ? 3 : 1;
+  if (I.fft_bytes < comps * one) {
+    cudaFree(I.fft_out);
+    I.fft_out = nullptr;
+    I.fft_bytes = 0;
+    CK(h, cudaMalloc(&I.fft_out, comps * one));
+    I.fft_bytes = comps * one;
+  }
+  if (I.fft_own && !I.fft_tw) {
+    std::vector<float2> tw((size_t)p.nx + p.ny + p.nz);
+    fft_twiddles(I.fft, tw.data());
+    CK(h, cudaMalloc(&I.fft_tw, sizeof(float2) * tw.size()));
+    CK(h, cudaMemcpyAsync(I.fft_tw, tw.data(), sizeof(float2) * tw.size(), cudaMemcpyHostToDevice, h->stream));
+    CK(h, cudaStreamSynchronize(h->stream));
+  }
+  if (!I.fft_own && !I.has_plan) {
     CKF(h, cufftPlan3d(&I.plan, p.nz, p.ny, p.nx, CUFFT_R2C));
     I.has_plan = true;
-    CK(h, cudaMalloc(&I.fft_out, sizeof(float) * 2 * (size_t)p.nz * p.ny * (p.nx / 2 + 1)));
+    CKF(h, cufftSetStream(I.plan, h->stream));
   }
-  CKF(h, cufftSetStream(I.plan, h->stream));
-  const int blocks = std::min(2 * h->num_sms, 1024);
+  const int blocks = I.fft_own ? I.fft.blocks[0] : bin_lines_blocks(p.nx, p.ny, p.nz, kmax, h->num_sms);
   const size_t need = (size_t)blocks * (kmax + 1) + (kmax + 1);
   if (need > h->spec_elems) {
     if (h->d_spec) cudaFree(h->d_spec);
     h->d_spec = nullptr;
+    h->spec_elems = 0;
     CK(h, cudaMalloc(&h->d_spec, need * sizeof(double)));
     h->spec_elems = need;
   }
   CK(h, cudaMemsetAsync(h->d_spec, 0, need * sizeof(double), h->stream));
-  for (int d = 0; d < 3; ++d) {
-    CKF(h, cufftExecR2C(I.plan, I.u + (size_t)d * I.ncell, static_cast<cufftComplex*>(I.fft_out)));
-    CK(h, launch_spec_bin(I.fft_out, p.nx, p.ny, p.nz, kmax, h->d_spec, blocks, h->stream));
+  float2* work = static_cast<float2*>(I.fft_out);
+  for (int d = 0; d < 3; d += comps) {
+    if (I.fft_own) {
+      CK(h, launch_fft_shells(I.u, I.fft, d, comps, kmax, I.fft_tw, work, h->d_spec, h->stream));
+    } else {
+      // the library wants its input on 8 bytes: components of an odd number of cells
+      // that start between are moved
+      float* in = I.u + (size_t)d * I.ncell;
+      if ((I.ncell & 1) && d) {
+        const int rc = ensure_scratch(h, sizeof(float) * (size_t)I.ncell);
+        if (rc != LBM_OK) return rc;
+        CK(h, cudaMemcpyAsync(h->d_scratch, in, sizeof(float) * (size_t)I.ncell, cudaMemcpyDeviceToDevice, h->stream));
+        in = static_cast<float*>(h->d_scratch);
+      }
+      CKF(h, cufftExecR2C(I.plan, in, reinterpret_cast<cufftComplex*>(work)));
+      CK(h, launch_bin_lines(work, p.nx, p.ny, p.nz, kmax, h->d_spec, blocks, h->stream));
+    }
   }
   double* Edev = h->d_spec + (size_t)blocks * (kmax + 1);
-  CK(h, launch_spec_finish(h->d_spec, blocks, kmax, Edev, h->stream));
+  const double ncell = (double)p.nx * p.ny * p.nz;
+  CK(h, launch_sum_cols(h->d_spec, blocks, kmax + 1, Edev, h->stream, 0.5 / (ncell * ncell)));
   CK(h, cudaMemcpyAsync(host_E, Edev, sizeof(double) * (kmax + 1), cudaMemcpyDeviceToHost, h->stream));
   CK(h, cudaStreamSynchronize(h->stream));
   I.spec_E.assign(host_E, host_E + kmax + 1);
@@ -670,6 +718,7 @@ void release(lbm_t h) {
     cudaFree(I.plane);
     cudaFree(I.hist);
     cudaFree(I.fft_out);
+    cudaFree(I.fft_tw);
     if (I.has_plan) cufftDestroy(I.plan);
   }
   cudaFree(h->d_desc);

@@ -1,6 +1,5 @@
 // Auxiliary kernels: initial equilibrium, canonical population access in the
-// AA layout, parity re-layout, the FP64 reduction finishers and the shell
-// binning of the energy spectrum.
+// AA layout, parity re-layout and the FP64 reduction finishers.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -189,76 +188,6 @@ __global__ void k_finish(const double* __restrict__ partials, int ninst, int gri
   }
 }
 
-// Exact integer shell: s with s^2 - s + 1 <= K <= s^2 + s (s - 1/2 <= sqrt K < s + 1/2).
-__device__ __forceinline__ int shell_of(long long K) {
-  long long r = (long long)sqrt((double)K);
-  while (r * r > K) --r;
-  while ((r + 1) * (r + 1) <= K) ++r;
-  return (int)(K > r * r + r ? r + 1 : r);
-}
-
-// shell_of for K < 2^24, where K is exact in FP32 and the FP32 square root is
-// within one of the integer root: no FP64 arithmetic (slow on this part).
-__device__ __forceinline__ int shell_of_small(int K) {
-  int r = (int)sqrtf((float)K);
-  while (r * r > K) --r;
-  while ((r + 1) * (r + 1) <= K) ++r;
-  return K > r * r + r ? r + 1 : r;
-}
-
-// A warp takes one (ky, kz) line of the half-spectrum at a time, lanes over kx
-// (no division per mode).  The shell does not decrease with kx, so the lanes
-// of one group of 32 modes that fall in one shell form a run: their FP32
-// energies are summed within the run (a segmented shuffle sum) and the run's
-// first lane adds the sum, scaled, to the block's FP64 shell total in shared
-// memory.
-__global__ void k_spec_bin(const float2* __restrict__ c, int nx, int ny, int nz, int kmax,
-                           double* __restrict__ partials) {
-  extern __shared__ double sh[];
-  for (int s = threadIdx.x; s <= kmax; s += blockDim.x) sh[s] = 0.0;
-  __syncthreads();
-  const int nxh = nx / 2 + 1;
-  const double ncell = (double)nx * ny * nz;
-  const double scale = 0.5 / (ncell * ncell);
-  const int lane = threadIdx.x & 31;
-  const int64_t lines = (int64_t)ny * nz;
-  const int64_t wstride = (int64_t)gridDim.x * (blockDim.x >> 5);
-  for (int64_t l = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); l < lines; l += wstride) {
-    const int kz = (int)(l / ny), ky = (int)(l - (int64_t)kz * ny);
-    const long long sy = ky <= ny / 2 ? ky : ky - ny;
-    const long long sz = kz <= nz / 2 ? kz : kz - nz;
-    const long long Kp = sy * sy + sz * sz;
-    const float2* row = c + l * nxh;
-    for (int x0 = 0; x0 < nxh; x0 += 32) {
-      const int kx = x0 + lane;
-      int s = kmax + 1;  // no contribution
-      float e = 0.f;
-      if (kx < nxh) {
-        const long long K = (long long)kx * kx + Kp;
-        const int sk = K < (1ll << 24) ? shell_of_small((int)K) : shell_of(K);
-        if (sk <= kmax) {
-          // the R2C half-spectrum holds each kx > 0 mode once for the pair
-          // (k, -k), except kx = 0 and the Nyquist plane kx = nx/2 (even nx)
-          const float2 v = row[kx];
-          s = sk;
-          e = ((kx == 0 || 2 * kx == nx) ? 1.f : 2.f) * (v.x * v.x + v.y * v.y);
-        }
-      }
-#pragma unroll
-      for (int off = 1; off < 32; off <<= 1) {
-        const float eo = __shfl_down_sync(0xffffffffu, e, off);
-        const int so = __shfl_down_sync(0xffffffffu, s, off);
-        if (lane + off < 32 && so == s) e += eo;
-      }
-      const int sp = __shfl_up_sync(0xffffffffu, s, 1);
-      if (s <= kmax && (lane == 0 || sp != s)) atomicAdd(&sh[s], scale * (double)e);
-    }
-  }
-  __syncthreads();
-  for (int s = threadIdx.x; s <= kmax; s += blockDim.x)
-    partials[(int64_t)blockIdx.x * (kmax + 1) + s] += sh[s];
-}
-
 // Column sums of a [rows][cols] table times `scale`, one warp per column in the fixed order
 // of k_finish (lane l adds rows l, l + 32, ...; then a shuffle tree).
 __global__ void k_sum_cols(const double* __restrict__ p, int rows, int cols, double scale,
@@ -372,17 +301,6 @@ cudaError_t launch_finish(const double* partials, int ninst, int grid, double* r
   const int warps_per_block = 256 / 32;
   const int blocks = std::max(1, std::min(1024, (ninst * kNP + warps_per_block - 1) / warps_per_block));
   return launch_kernel(k_finish, blocks, 256, 0, st, partials, ninst, grid, results, ring, seq, cap, err);
-}
-
-cudaError_t launch_spec_bin(const void* coeffs, int nx, int ny, int nz, int kmax,
-                            double* partials, int blocks, cudaStream_t st) {
-  return launch_kernel(k_spec_bin, blocks, kAuxThreads, (size_t)(kmax + 1) * sizeof(double), st,
-                       static_cast<const float2*>(coeffs), nx, ny, nz, kmax, partials);
-}
-
-cudaError_t launch_spec_finish(const double* partials, int blocks, int kmax, double* E,
-                               cudaStream_t st) {
-  return launch_sum_cols(partials, blocks, kmax + 1, E, st);
 }
 
 cudaError_t launch_sum_cols(const double* partials, int rows, int cols, double* out,

@@ -110,12 +110,6 @@ cudaError_t launch_relayout_pair(const InstDesc& d, int precision, bool from_odd
 cudaError_t launch_finish(const double* partials, int ninst, int grid, double* results,
                           double* ring, unsigned long long* seq, int cap, uint32_t* err,
                           cudaStream_t st);
-// Shell sums of |u_hat|^2 / ncell^2 from an R2C spectrum [nz][ny][nx/2+1]:
-// partials [blocks][kmax + 1] (accumulated onto), then summed by launch_spec_finish.
-cudaError_t launch_spec_bin(const void* coeffs, int nx, int ny, int nz, int kmax,
-                            double* partials, int blocks, cudaStream_t st);
-cudaError_t launch_spec_finish(const double* partials, int blocks, int kmax, double* E,
-                               cudaStream_t st);
 // out[c] = scale * sum over rows of partials[rows][cols].
 cudaError_t launch_sum_cols(const double* partials, int rows, int cols, double* out,
                             cudaStream_t st, double scale = 1.0);
