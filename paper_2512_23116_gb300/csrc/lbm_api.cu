@@ -34,6 +34,8 @@ using namespace lbm;
 constexpr int kRingCap = 1024;
 constexpr int kMinHistWindow = 256;  // fewer histogram bins than this in shared memory: all global
 constexpr int64_t kChunkCells = 4 << 20;
+constexpr size_t kDirectBytes = 24 << 20;     // populations up to this size: direct kernel, no others timed
+constexpr size_t kDirectMaxBytes = 40 << 20;  // and up to this size (FP32): the direct kernel among others
 constexpr size_t kFftBatchBytes = 192 << 20;  // three half spectra (256^3) transformed together
 constexpr double kPi = 3.14159265358979323846;
 
@@ -51,6 +53,7 @@ struct Inst {
   double hist_max = 0.02;
   int rows = 1;
   int64_t tile_begin = 0, tile_end = 0;
+  int64_t chunk_begin = 0, chunk_end = 0;
   // lazily allocated diagnostic buffers
   float* u = nullptr;       // [3][ncell]
   float* aux = nullptr;     // [3][ncell]
@@ -90,7 +93,8 @@ struct lbm_s {
   std::vector<Inst> inst;
   InstDesc* d_desc = nullptr;
   std::vector<InstDesc> h_desc;
-  int64_t total_tiles = 0;
+  int64_t total_tiles = 0, total_chunks = 0;
+  int chunk = 256;     // cells of a direct-kernel chunk: its threads per block
   int64_t t = 0;
   uint64_t version = 1;  // bumped by every call that changes the populations
   // kernel configuration
@@ -251,15 +255,15 @@ void clear_graphs(lbm_t h) {
   h->graphs.clear();
 }
 
-// Blocks of the read-only statistics pass: the direct kernel (256 threads) at
-// full occupancy.
+// Blocks of the read-only statistics pass: the direct kernel at full occupancy.
 int diag_grid(lbm_t h) {
-  return h->num_sms * std::max(1, direct_max_blocks_per_sm(h->precision, 256));
+  return h->num_sms * std::max(1, direct_max_blocks_per_sm(h->precision, h->chunk));
 }
 
 // Tile decomposition for the current configuration; uploads the descriptor table.
 int build_tiles(lbm_t h) {
-  int64_t tile = 0;
+  int64_t tile = 0, chunk = 0;
+  h->chunk = h->kind == 1 ? h->threads : 256;
   h->h_desc.resize(h->inst.size());
   for (size_t i = 0; i < h->inst.size(); ++i) {
     Inst& I = h->inst[i];
@@ -280,6 +284,9 @@ int build_tiles(lbm_t h) {
     I.tile_begin = tile;
     tile += (int64_t)tpp * p.nz;
     I.tile_end = tile;
+    I.chunk_begin = chunk;
+    chunk += (I.ncell + h->chunk - 1) / h->chunk;
+    I.chunk_end = chunk;
     InstDesc& d = h->h_desc[i];
     d.f = I.f;
     d.fx_of_y = I.tables;
@@ -314,9 +321,12 @@ int build_tiles(lbm_t h) {
     d.tiles_per_plane = tpp;
     d.tile_begin = I.tile_begin;
     d.tile_end = I.tile_end;
+    d.chunk_begin = I.chunk_begin;
+    d.chunk_end = I.chunk_end;
     d.f_elems = (int64_t)(I.f_bytes / h->esize);
   }
   h->total_tiles = tile;
+  h->total_chunks = chunk;
   CK(h, cudaMemcpyAsync(h->d_desc, h->h_desc.data(), sizeof(InstDesc) * h->h_desc.size(),
                         cudaMemcpyHostToDevice, h->stream));
   // partials for every block and instance
@@ -337,8 +347,10 @@ LaunchArgs base_args(lbm_t h) {
   LaunchArgs la{};
   la.insts = h->d_desc;
   la.ninst = (int)h->inst.size();
+  la.one = h->h_desc[0];
   la.tile_lo = 0;
-  la.tile_hi = h->total_tiles;
+  la.tile_hi = h->kind == 2 ? h->total_tiles : h->total_chunks;
+  for (const Inst& I : h->inst) la.wide = la.wide || I.f_bytes >= ((size_t)1 << 32);
   la.precision = h->precision;
   la.sa.partials = h->d_partials;
   la.sa.grid = h->grid;
@@ -540,7 +552,14 @@ int diag_pass(lbm_t h, int i, bool want_u, bool want_aux, int plane_axis, int pl
   }
   if (grid == 0) {
     LaunchArgs ld = la;
-    ld.threads = 256;
+    ld.threads = h->chunk;
+    ld.tile_lo = I.chunk_begin;
+    ld.tile_hi = I.chunk_end;
+    if (plane_only) {  // the chunks that hold cells of the plane
+      const int64_t pc = (int64_t)I.p.nx * I.p.ny;
+      ld.tile_lo = I.chunk_begin + plane_index * pc / h->chunk;
+      ld.tile_hi = I.chunk_begin + ((plane_index + 1) * pc + h->chunk - 1) / h->chunk;
+    }
     ld.grid = grid = diag_grid(h);
     ld.sa.grid = ld.grid;
     CK(h, launch_step_direct(ld, h->stream));
@@ -864,22 +883,50 @@ int64_t max_row_stage_bytes(lbm_t h) {
   return m;
 }
 
-double time_candidate(lbm_t h, int steps) {
+// Milliseconds of `steps` plain steps of the current configuration.  Small
+// lattices (graph) are timed as they will run, replayed from a captured graph: launched
+// one by one, their steps take as long as the host takes to launch them,
+// whatever the kernel.
+double time_candidate(lbm_t h, int steps, bool graph) {
   cudaEvent_t a, b;
   cudaEventCreate(&a);
   cudaEventCreate(&b);
   const bool g = h->use_graphs;
-  h->use_graphs = false;
   const int saved_every = h->stats_every;
   h->stats_every = 0;
-  enqueue_steps(h, 0, 2);  // warm-up
-  cudaEventRecord(a, h->stream);
-  int rc = enqueue_steps(h, 0, steps);
-  cudaEventRecord(b, h->stream);
-  cudaError_t e = cudaEventSynchronize(b);
+  cudaGraphExec_t ex = nullptr;
+  int rc = LBM_OK;
+  if (graph && g) {
+    cudaGraph_t cg = nullptr;
+    const bool pending = cudaPeekAtLastError() != cudaSuccess;  // the caller's, left alone
+    cudaError_t e = cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal);
+    if (e == cudaSuccess) {
+      rc = enqueue_steps(h, 0, steps);
+      e = cudaStreamEndCapture(h->stream, &cg);
+    }
+    if (rc == LBM_OK && e == cudaSuccess) e = cudaGraphInstantiate(&ex, cg, 0);
+    if (cg) cudaGraphDestroy(cg);
+    if ((rc != LBM_OK || e != cudaSuccess) && !pending) (void)cudaGetLastError();
+    if (e != cudaSuccess) ex = nullptr;
+  }
+  h->use_graphs = false;
+  cudaError_t e = cudaSuccess;
+  if (ex) {
+    e = cudaGraphLaunch(ex, h->stream);  // warm-up
+    cudaEventRecord(a, h->stream);
+    if (e == cudaSuccess) e = cudaGraphLaunch(ex, h->stream);
+    cudaEventRecord(b, h->stream);
+  } else if (rc == LBM_OK) {
+    enqueue_steps(h, 0, 2);  // warm-up
+    cudaEventRecord(a, h->stream);
+    rc = enqueue_steps(h, 0, steps);
+    cudaEventRecord(b, h->stream);
+  }
+  if (e == cudaSuccess && rc == LBM_OK) e = cudaEventSynchronize(b);
   float ms = 0.f;
   if (rc == LBM_OK && e == cudaSuccess) cudaEventElapsedTime(&ms, a, b);
   else ms = 1e30f;
+  if (ex) cudaGraphExecDestroy(ex);
   cudaEventDestroy(a);
   cudaEventDestroy(b);
   h->use_graphs = g;
@@ -931,9 +978,30 @@ int choose_config(lbm_t h, const lbm_params& p0) {
     c.layout = lay_fixed;
     return apply_candidate(h, c);
   }
-  if (requested_kind == 1 || requested_kind == 0)
-    cands.push_back({1, 256, 0, 0, requested_rows, 0, lay_fixed});
-  if ((requested_kind == 2 || requested_kind == 0) && tma_ok) {
+  size_t bytes = 0;
+  for (const Inst& I : h->inst) bytes += I.f_bytes;
+  // Lattices deep inside the L2 cache always step fastest with the direct kernel (a TMA
+  // block sees a tile or two per step, all of it pipeline fill and drain): FP32 32^3
+  // 2.1 against 5.1 us, 64^3 (20 MB) 6.1 against 8.6; FP16 80^3 (19 MB) 9.7 against 11.4.
+  // In FP32 both are timed up to kDirectMaxBytes (80^3, 39 MB: 10.6 against 12.5); above,
+  // the two are level while the cache is the lattice's own (100^3, 76 MB: 19.9
+  // against 20.3) and the TMA kernel is ahead once it is shared or outgrown (three
+  // lattices of 100^3 stepped in turn: 22.8 against 27.5 us; three of 96^3 in FP16, 34 MB
+  // each: 9.0 against 10.0).
+  // The two kernels give the same bits but for the self-consistent strain (strain_mode 1),
+  // whose last bit differs; in 16-bit storage that grows to a spacing of the storage
+  // format, so such handles stay with the TMA kernel whatever their size.
+  bool alike = h->precision == LBM_FP32;
+  if (!alike) {
+    alike = true;
+    for (const Inst& I : h->inst) alike = alike && I.p.strain_mode == 0;
+  }
+  const bool direct_only = requested_kind == 0 && alike && bytes <= kDirectBytes;
+  const bool want_direct =
+      requested_kind == 1 || (requested_kind == 0 && (direct_only || (h->precision == LBM_FP32 && bytes <= kDirectMaxBytes) || !tma_ok));
+  if (want_direct)
+    for (int th : {64, 128, 256}) cands.push_back({1, th, 0, 0, requested_rows, 0, lay_fixed});
+  if ((requested_kind == 2 || requested_kind == 0) && !direct_only && tma_ok) {
     // a stage holds R x-lines of every population (exact multiples of one row stage)
     const int row_opts[] = {1, 2, 3, 4, 6, 8, 12, 16};
     const int stage_opts[] = {2, 3, 4};
@@ -998,6 +1066,7 @@ int choose_config(lbm_t h, const lbm_params& p0) {
       cands.push_back(c);
     }
   }
+  if (cands.empty() && requested_kind == 0) cands.push_back({1, 256, 0, 0, requested_rows, 0, lay_fixed});
   if (cands.empty())
     return fail(h, LBM_ERR_UNSUPPORTED, "no kernel configuration fits this lattice");
   if (cands.size() == 1) return apply_candidate(h, cands[0]);
@@ -1009,7 +1078,7 @@ int choose_config(lbm_t h, const lbm_params& p0) {
   Candidate bc = cands[0];
   for (const Candidate& c : cands) {
     if (apply_candidate(h, c) != LBM_OK) continue;
-    const double ms = time_candidate(h, steps);
+    const double ms = time_candidate(h, steps, direct_only);
     if (ms < best) {
       best = ms;
       bc = c;

@@ -30,6 +30,8 @@ struct InstDesc {
   int32_t tiles_per_plane; // ceil(ny / rows)
   int64_t tile_begin;      // first global tile of the instance
   int64_t tile_end;        // one past the last
+  int64_t chunk_begin;     // the direct kernel's chunks of consecutive cells: first of the instance,
+  int64_t chunk_end;       // one past the last
   int64_t f_elems;         // storage elements of the population array (bounds checks)
 };
 

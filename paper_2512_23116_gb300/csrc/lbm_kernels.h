@@ -27,16 +27,36 @@ inline cudaError_t launch_kernel(void (*kernel)(P...), dim3 grid, dim3 block, si
   return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
 }
 
+// The same as a programmatic dependent of the kernel before it in the stream (which
+// it waits for itself, by griddepcontrol.wait).
+template <typename... P, typename... A>
+inline cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                                    A&&... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+}
+
 struct LaunchArgs {
   const InstDesc* insts;   // device table
+  InstDesc one;            // its first entry (the only one when ninst == 1)
   int ninst;
-  int64_t tile_lo, tile_hi;
+  int64_t tile_lo, tile_hi; // tiles of the TMA kernel, chunks of `threads` cells of the direct one
   int precision;           // 0 fp32, 1 fp16, 2 bf16
   bool odd;                // AA parity of the step (time t odd)
   int mode;                // MODE_STEP | MODE_STEP_STATS | MODE_DIAG
   StatsArgs sa;
   DiagOut dout;
   int grid, threads;
+  bool wide;               // direct kernel: some population array is 4 GB or more (64-bit offsets)
   // TMA kernel configuration
   int stages;
   int slot_bytes;          // shared-memory slot per population segment: kSlot3, kSlot2, kSlot2h, or the runtime

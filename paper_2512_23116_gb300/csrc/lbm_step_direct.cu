@@ -5,8 +5,26 @@
 // writes f*_a to slot a of x + c_a.  Each cell reads exactly the locations it
 // writes, so all cells of a step are independent (Eq. mrt_les_guo, with
 // periodic streaming of Sec. 3.1).  One thread per cell, plain coalesced
-// loads and stores; the grid walks tiles of `rows` x-lines.
+// loads and stores.
+//
+// Work is dealt out in chunks of blockDim.x consecutive cells (x fastest, rows and
+// planes running on), so no thread idles at the end of a row or a tile; the
+// coordinates advance from chunk to chunk by additions.  The location that f*_a goes to
+// is the one f_opp(a) came from, so 19 offsets serve loads and stores; they are
+// 32-bit for arrays below 4 GB (WIDE = false).
+//
+// What bounds it: the L2 cache.  With the collision taken out a step of 64^3 takes
+// 5.7 of its 6.1 us and one of 100^3 18.5 of 19.9 (9 TB/s; the odd step's x-shifted
+// slots cost 2-3 us of that in partly written sectors); prefetching the next
+// cell, into registers or by asynchronous copies, made it slower.  Below that it is
+// latency: launches and the first loads, which the launch parameter `one`, 32-bit
+// divisions and dependent launches shorten.  A step of 16^3 1.5 us, 32^3 2.1 (5.1 before,
+// the TMA kernel's; 5.8 for one-thread-per-cell tiles of whole rows with 64-bit offsets),
+// 48^3 3.5 (6.0), 64^3 6.1 (8.6), 80^3 10.6 (12.5); beyond ~100^3 the TMA kernel is ahead
+// (128^3: 54 against 61).
 #include <cuda_runtime.h>
+
+#include <type_traits>
 
 #include "lbm_device.cuh"
 #include "lbm_kernels.h"
@@ -16,11 +34,89 @@ namespace lbm {
 
 constexpr int kSmemHistBins = 12000;  // (bins + 1) * 4 bytes below 48 KB
 
-template <typename T, bool ODD, int MODE>
+namespace {
+
+// What a thread keeps of the instance it is in.
+template <typename I>
+struct CellWalk {
+  int64_t end;             // one past the instance's last chunk
+  int nx, ny, nz;
+  int x, y, z;             // the thread's cell
+  int dx, dy, dz;          // from one of the block's chunks to its next
+  I slot, row, plane;      // strides (values)
+  bool grouped;
+  __device__ __forceinline__ void enter(const InstDesc& d, int64_t t, int64_t stride) {
+    end = d.chunk_end;
+    nx = d.nx;
+    ny = d.ny;
+    nz = d.nz;
+    slot = (I)d.slot_stride;
+    row = (I)d.row_stride;
+    plane = (I)d.plane_stride;
+    grouped = d.slot_grouped != 0;
+    // cells and strides fit 32 bits with 32-bit offsets
+    using U = typename std::conditional<sizeof(I) == 4, uint32_t, int64_t>::type;
+    const U plane_cells = (U)nx * (U)ny;
+    const U c = (U)(t - d.chunk_begin) * blockDim.x + threadIdx.x, s = (U)stride * blockDim.x;
+    z = (int)(c / plane_cells);
+    const U r = c - (U)z * plane_cells;
+    y = (int)(r / (U)nx);
+    x = (int)(r - (U)y * (U)nx);
+    dz = (int)(s / plane_cells);
+    const U q = s - (U)dz * plane_cells;
+    dy = (int)(q / (U)nx);
+    dx = (int)(q - (U)dy * (U)nx);
+  }
+  __device__ __forceinline__ void next() {
+    x += dx;
+    y += dy;
+    z += dz;
+    if (x >= nx) {
+      x -= nx;
+      ++y;
+    }
+    if (y >= ny) {
+      y -= ny;
+      ++z;
+    }
+  }
+};
+
+// Offset of what the cell reads as f_a (values): the even step's slot a of the cell, the
+// odd step's slot opp(a) of the cell at -c_a.  f*_a goes to the location of opp(a).
+template <typename I, bool ODD>
+__device__ __forceinline__ void offsets(const CellWalk<I>& w, I (&o)[19]) {
+  if (!ODD) {
+    const I c = (I)w.z * w.plane + (I)w.y * w.row + (I)w.x;
+#pragma unroll
+    for (int a = 0; a < 19; ++a) o[a] = c + (I)(w.grouped ? gpos(a) : a) * w.slot;
+  } else {
+    const I xs[3] = {(I)wrap_inc(w.x, w.nx), (I)w.x, (I)wrap_dec(w.x, w.nx)};  // by cx + 1
+    const I ys[3] = {(I)wrap_inc(w.y, w.ny) * w.row, (I)w.y * w.row, (I)wrap_dec(w.y, w.ny) * w.row};
+    const I zs[3] = {(I)wrap_inc(w.z, w.nz) * w.plane, (I)w.z * w.plane, (I)wrap_dec(w.z, w.nz) * w.plane};
+#pragma unroll
+    for (int a = 0; a < 19; ++a)
+      o[a] = (zs[cz(a) + 1] + ys[cy(a) + 1]) + (xs[cx(a) + 1] + (I)(w.grouped ? gpos(opp(a)) : opp(a)) * w.slot);
+  }
+}
+
+}  // namespace
+
+// Dependent launches: the next step's blocks may start, and read their launch
+// parameters, while this step's last blocks still run; nothing of the populations is
+// touched before dependency_wait, which returns when the step before has completed
+// and its writes are visible.
+__device__ __forceinline__ void dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void dependents_may_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// ONE: a single instance, described by the launch parameter `one` (the table costs a chain of
+// dependent loads before the first population can be read).
+template <typename T, bool ODD, int MODE, bool WIDE, bool ONE>
 __global__ void __launch_bounds__(256, 2)
-k_step_direct(const InstDesc* __restrict__ insts, int ninst, int64_t tile_lo, int64_t tile_hi,
-              StatsArgs sa, DiagOut dout) {
+k_step_direct(const InstDesc* __restrict__ insts, int ninst, int64_t chunk_lo, int64_t chunk_hi,
+              StatsArgs sa, DiagOut dout, const __grid_constant__ InstDesc one) {
   using S = Storage<T>;
+  using I = typename std::conditional<WIDE, int64_t, uint32_t>::type;
   extern __shared__ uint32_t shist[];
   // theta histogram in shared memory when it fits the default 48 KB, else
   // straight into the global counts
@@ -35,87 +131,72 @@ k_step_direct(const InstDesc* __restrict__ insts, int ninst, int64_t tile_lo, in
   uint32_t* const hist_sm = use_hist ? shist : nullptr;
   const int hist_win = use_hist ? dout.hist_bins + 1 : 0;
   uint32_t* const hist_gl = use_hist ? nullptr : dout.hist;
-  int cur = -1, hint = 0;
-  for (int64_t t = tile_lo + blockIdx.x; t < tile_hi; t += gridDim.x) {
-    const int ii = find_instance(insts, ninst, t, cur < 0 ? hint : cur);
-    hint = ii;
-    if (MODE != MODE_STEP && ii != cur) {
-      if (cur >= 0)
-        block_flush(acc, sa.partials + ((int64_t)cur * sa.grid + blockIdx.x) * kNP, blockDim.x, 0);
-      acc.reset();
-      cur = ii;
-    }
-    const InstDesc& d = insts[ii];
-    const int nx = d.nx, ny = d.ny, nz = d.nz;
-    const int64_t ps = d.slot_stride, pls = d.plane_stride, rs = d.row_stride;
-    const bool grouped = d.slot_grouped != 0;
-    // position of cell (x, y, z) within a population slot; offset of slot a
-    auto at = [pls, rs](int x, int y, int z) { return z * pls + y * rs + x; };
-    auto slot = [ps, grouped](int a) { return (grouped ? gpos(a) : a) * ps; };
-    const int64_t local = t - d.tile_begin;
-    const int z = (int)(local / d.tiles_per_plane);
-    const int y0 = (int)(local - (int64_t)z * d.tiles_per_plane) * d.rows;
-    const int rows = min(d.rows, ny - y0);
-    const int ncell = rows * nx;
-    T* __restrict__ fb = static_cast<T*>(d.f);
-    const int zm = wrap_dec(z, nz), zp = wrap_inc(z, nz);
-    const float Fy = (in_bounds(z >= 0 && z < nz) ? d.fy_of_z[z] : 0.f) + d.fconst[1];
-    const float nu0 = d.nu0, s_nu0 = d.s_nu0, C = d.C;
-    const int dr = blockDim.x / nx, dx = blockDim.x - dr * nx;  // a pass of blockDim.x cells
-    int r = threadIdx.x / nx, x = threadIdx.x - r * nx;
-    for (int c = threadIdx.x; c < ncell; c += blockDim.x) {
-      const int y = y0 + r;
-      const int ym = wrap_dec(y, ny), yp = wrap_inc(y, ny);
-      const int xm = wrap_dec(x, nx), xp = wrap_inc(x, nx);
-      float f[19];
-      if (!ODD) {
-        const int64_t o = at(x, y, z);
-#pragma unroll
-        for (int a = 0; a < 19; ++a) {
-          const int64_t i = slot(a) + o;
-          f[a] = in_bounds(i >= 0 && i < d.f_elems) ? S::load(fb + i) : 0.f;
-        }
-      } else {
-#pragma unroll
-        for (int a = 0; a < 19; ++a) {
-          const int xs = cx(a) > 0 ? xm : (cx(a) < 0 ? xp : x);
-          const int ys = cy(a) > 0 ? ym : (cy(a) < 0 ? yp : y);
-          const int zs = cz(a) > 0 ? zm : (cz(a) < 0 ? zp : z);
-          const int64_t i = slot(opp(a)) + at(xs, ys, zs);
-          f[a] = in_bounds(i >= 0 && i < d.f_elems) ? S::load(fb + i) : 0.f;
-        }
+  int cur = -1;
+  CellWalk<I> w;
+  w.end = -1;
+  T* __restrict__ fb = nullptr;
+  const float *fx = nullptr, *fy = nullptr, *fz = nullptr;
+  float cfx = 0.f, cfy = 0.f, cfz = 0.f, nu0 = 0.f, s_nu0 = 0.f, C = 0.f;
+  int smode = 0;
+  if (MODE == MODE_STEP) dependents_may_start();
+  bool waited = MODE != MODE_STEP;
+  for (int64_t t = chunk_lo + blockIdx.x; t < chunk_hi; t += gridDim.x) {
+    if (t >= w.end) {
+      const int ii = ONE ? 0 : find_chunk_instance(insts, ninst, t, cur < 0 ? 0 : cur);
+      if (MODE != MODE_STEP) {
+        if (cur >= 0)
+          block_flush(acc, sa.partials + ((int64_t)cur * sa.grid + blockIdx.x) * kNP, blockDim.x, 0);
+        acc.reset();
       }
-      const float Fx = (in_bounds(y >= 0 && y < ny) ? d.fx_of_y[y] : 0.f) + d.fconst[0];
-      const float Fz = (in_bounds(x >= 0 && x < nx) ? d.fz_of_x[x] : 0.f) + d.fconst[2];
+      cur = ii;
+      const InstDesc& d = ONE ? one : insts[ii];
+      w.enter(d, t, gridDim.x);
+      fb = static_cast<T*>(d.f);
+      fx = d.fx_of_y;
+      fy = d.fy_of_z;
+      fz = d.fz_of_x;
+      cfx = d.fconst[0];
+      cfy = d.fconst[1];
+      cfz = d.fconst[2];
+      nu0 = d.nu0;
+      s_nu0 = d.s_nu0;
+      C = d.C;
+      smode = d.strain_mode;
+    } else {
+      w.next();
+    }
+    if (!waited) {
+      dependency_wait();
+      waited = true;
+    }
+    // one copy of the cell's work per strain mode, a constant in each, as in the TMA
+    // kernel: the compiler then contracts the same operations, and the two kernels give
+    // the same bits
+    auto cell = [&](auto mode) __attribute__((always_inline)) {
+      I o[19];
+      offsets<I, ODD>(w, o);
+      float f[19];
+#pragma unroll
+      for (int a = 0; a < 19; ++a)
+        f[a] = in_bounds((int64_t)o[a] >= 0 && (int64_t)o[a] < (ONE ? one : insts[cur]).f_elems) ? S::load(fb + o[a]) : 0.f;
+      const float Fx = fx[w.y] + cfx, Fy = fy[w.z] + cfy, Fz = fz[w.x] + cfz;
       CellDiag g;
-      mrt_collide(f, Fx, Fy, Fz, nu0, s_nu0, C, g, d.strain_mode);
+      mrt_collide(f, Fx, Fy, Fz, nu0, s_nu0, C, g, decltype(mode)::value);
       if (MODE != MODE_DIAG) {
-        if (!ODD) {
-          const int64_t o = at(x, y, z);
 #pragma unroll
-          for (int a = 0; a < 19; ++a) {
-            const int64_t i = slot(opp(a)) + o;
-            if (in_bounds(i >= 0 && i < d.f_elems)) fb[i] = S::pack(f[a]);
-          }
-        } else {
-#pragma unroll
-          for (int a = 0; a < 19; ++a) {
-            const int xd = cx(a) > 0 ? xp : (cx(a) < 0 ? xm : x);
-            const int yd = cy(a) > 0 ? yp : (cy(a) < 0 ? ym : y);
-            const int zd = cz(a) > 0 ? zp : (cz(a) < 0 ? zm : z);
-            const int64_t i = slot(a) + at(xd, yd, zd);
-            if (in_bounds(i >= 0 && i < d.f_elems)) fb[i] = S::pack(f[a]);
-          }
-        }
+        for (int a = 0; a < 19; ++a)
+          if (in_bounds((int64_t)o[opp(a)] >= 0 && (int64_t)o[opp(a)] < (ONE ? one : insts[cur]).f_elems))
+            fb[o[opp(a)]] = S::pack(f[a]);
       }
       if (MODE != MODE_STEP) acc.add(g, Fx, Fy, Fz, C);
-      if (MODE == MODE_DIAG) diag_write(dout, g, x, y, z, nx, ny, nz, hist_sm, 0, hist_win, hist_gl, run);
-      x += dx;
-      r += dr;
-      if (x >= nx) {
-        x -= nx;
-        r += 1;
-      }
+      if (MODE == MODE_DIAG)
+        diag_write(dout, g, w.x, w.y, w.z, w.nx, w.ny, w.nz, hist_sm, 0, hist_win, hist_gl, run);
+    };
+    if (w.z < w.nz) {  // the last chunk of an instance may run past its cells
+      if (smode == 1)
+        cell(std::integral_constant<int, 1>{});
+      else
+        cell(std::integral_constant<int, 0>{});
     }
     if (MODE != MODE_STEP) acc.fold_if_full();
   }
@@ -133,11 +214,18 @@ k_step_direct(const InstDesc* __restrict__ insts, int ninst, int64_t tile_lo, in
 
 template <typename T, bool ODD, int MODE>
 static cudaError_t launch_direct_t(const LaunchArgs& la, cudaStream_t st) {
+  if constexpr (MODE == MODE_STEP) {
+    if (la.ninst == 1 && !la.wide)
+      return launch_dependent(k_step_direct<T, ODD, MODE, false, true>, la.grid, la.threads, 0, st, la.insts, la.ninst,
+                              la.tile_lo, la.tile_hi, la.sa, la.dout, la.one);
+    return launch_dependent(la.wide ? k_step_direct<T, ODD, MODE, true, false> : k_step_direct<T, ODD, MODE, false, false>,
+                            la.grid, la.threads, 0, st, la.insts, la.ninst, la.tile_lo, la.tile_hi, la.sa, la.dout, la.one);
+  }
   const size_t smem = (MODE == MODE_DIAG && la.dout.hist && la.dout.hist_bins < kSmemHistBins)
                           ? (size_t)(la.dout.hist_bins + 1) * 4
                           : 0;
-  return launch_kernel(k_step_direct<T, ODD, MODE>, la.grid, la.threads, smem, st, la.insts, la.ninst,
-                       la.tile_lo, la.tile_hi, la.sa, la.dout);
+  return launch_kernel(la.wide ? k_step_direct<T, ODD, MODE, true, false> : k_step_direct<T, ODD, MODE, false, false>,
+                       la.grid, la.threads, smem, st, la.insts, la.ninst, la.tile_lo, la.tile_hi, la.sa, la.dout, la.one);
 }
 
 template <typename T>
@@ -165,9 +253,9 @@ int direct_max_blocks_per_sm(int precision, int threads) {
   int n = 0;
   cudaError_t e = cudaErrorInvalidValue;
   switch (precision) {
-    case 0: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_step_direct<float, true, MODE_STEP>, threads, 0); break;
-    case 1: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_step_direct<__half, true, MODE_STEP>, threads, 0); break;
-    case 2: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_step_direct<__nv_bfloat16, true, MODE_STEP>, threads, 0); break;
+    case 0: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_step_direct<float, true, MODE_STEP, false, false>, threads, 0); break;
+    case 1: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_step_direct<__half, true, MODE_STEP, false, false>, threads, 0); break;
+    case 2: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_step_direct<__nv_bfloat16, true, MODE_STEP, false, false>, threads, 0); break;
   }
   return e == cudaSuccess ? n : 0;
 }

@@ -23,14 +23,14 @@
 //    the exact increments.  This part executes 2 FP64 operations per clock and
 //    SM against 128 in FP32, so increments, powers and running sums are kept as
 //    unevaluated sums of FP32 words (Dekker 1971; Knuth's two-sum, products with
-//    an FMA for the remainder).  Against long double sums it is off by 1-4e-16
-//    of S_2, S_4, S_6 and 1-8e-18 of <|d|^3>, <|d|^5> on 50x61x77 to 100^3, where
-//    the FP64 loop left 3-7e-16 and 4e-18-6e-17.  Each tile scales its increments
+//    an FMA for the remainder).  Against quadruple-precision sums it is off by 1-2e-16
+//    of S_2, S_4, S_6 and 1-7e-18 of <|d|^3>, <|d|^5> on lattices of 1.0e5 to 1.4e6 cells,
+//    where the FP64 loop left 3-7e-16 and 1e-18-2e-17.  Each tile scales its increments
 //    by a power of two so that neither the sixth power nor its low words leave the
 //    FP32 range; a tile whose values do not allow that (infinities, NaN, extreme
-//    exponents) is summed in FP64.  Bound by issue: ~170 FP32 operations an
+//    exponents) is summed in FP64.  Bound by issue: ~180 FP32 operations an
 //    increment.  12 separations at 160^3: 4.43 ms (one FP64 pass over global memory
-//    per separation, at the FP64 rate) -> 0.87 ms.
+//    per separation, at the FP64 rate) -> 0.94 ms.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -50,8 +50,8 @@ constexpr int kRunMax = 64;     // cells a lane sums before the warp reduces
 constexpr int kWarpsMax = 8;
 // Lattices below this many cells are summed in FP64 terms: on 7,680 cells the
 // roundings of the three-word even powers left 1.7-2.9e-16 of S_2, S_4, S_6 where
-// FP64 left 0.7-1.5e-16; from 96,000 cells on they leave less (1.9e-16 against
-// 4-5e-16), and the two cost the same time only where both are short of work.
+// FP64 left 0.7-1.5e-16; from 96,000 cells on they leave less (1e-16 against
+// 4-5e-16).
 constexpr int64_t kWordsCells = 1 << 16;
 constexpr int kSmemMax = 225 * 1024;  // dynamic shared memory of a block, beside the few static words
 
@@ -126,16 +126,12 @@ __device__ __forceinline__ Words sqr_short(const Words& a) {
   return c;
 }
 
-// Running sums of (d, d^2, ..., d^6) of one separation.  The low words of d^2 are
-// summed apart from the remainders of its sum (`low2`): their sum rounds with a
-// bias when increments have few significant bits.
+// Running sums of (d, d^2, ..., d^6) of one separation.
 struct PowerSums {
   Words s[6];
-  float low2;
   __device__ __forceinline__ void reset() {
 #pragma unroll
     for (int k = 0; k < 6; ++k) s[k] = {0.f, 0.f, 0.f};
-    low2 = 0.f;
   }
   // d = (a - b) times `scale`, a power of two: exact in two words
   __device__ __forceinline__ void add(float a, float b, float scale) {
@@ -144,8 +140,7 @@ struct PowerSums {
     const Words d = {__fmul_rn(r, scale), __fmul_rn(e, scale), 0.f};
     const Words q = sqr_full(d), c = mul_full(q, d);
     add_full(s[0], d);
-    add_short(s[1], {q.h, 0.f, q.m});
-    low2 = __fadd_rn(low2, q.l);
+    add_full(s[1], q);  // its low words have few bits, whose sum would round with a bias
     add_full(s[2], c);
     add_short(s[3], sqr_short(q));
     add_full(s[4], mul_full(c, q));
@@ -178,8 +173,6 @@ __device__ __forceinline__ double warp_sums(const PowerSums (&v)[2], int lane) {
   Words a[16];
 #pragma unroll
   for (int i = 0; i < 16; ++i) a[i] = i < 12 ? v[i / 6].s[i % 6] : Words{0.f, 0.f, 0.f};
-  add_full(a[1], {0.f, v[0].low2, 0.f});
-  add_full(a[7], {0.f, v[1].low2, 0.f});
 #pragma unroll
   for (int s = 16; s > 0; s >>= 1) {
     const bool up = (lane & s) != 0;
