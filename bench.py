@@ -83,7 +83,7 @@ def traffic_per_update(kernel_digest: str, storage: str = "fp32"):
 
 # Sources that define the step kernel k_step_tma and what it computes per cell.
 STEP_KERNEL_SOURCES = ("lbm_device.cuh", "lbm_internal.h", "lbm_kernels.h", "lbm_reduce.cuh",
-                       "lbm_step_tma.cu")
+                       "lbm_step_tma.cu", "lbm_words.cuh")
 
 
 def _code_only(text: str) -> str:

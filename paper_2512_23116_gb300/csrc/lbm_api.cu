@@ -511,7 +511,10 @@ int diag_pass(lbm_t h, int i, bool want_u, bool want_aux, int plane_axis, int pl
   la.dout.hist = want_hist ? I.hist : nullptr;
   la.dout.hist_bins = I.hist_bins;
   la.dout.hist_scale = (float)(I.hist_bins / I.hist_max);
-  CK(h, cudaMemsetAsync(h->d_partials, 0, h->partials_elems * sizeof(double), h->stream));
+  if (plane_only)
+    la.sa.partials = nullptr;
+  else
+    CK(h, cudaMemsetAsync(h->d_partials, 0, h->partials_elems * sizeof(double), h->stream));
   // The TMA kernel's read-only variant when the handle runs the TMA kernel
   // (its copy pipeline keeps the loads in flight during the collision
   // arithmetic; the theta histogram goes behind the Fz table in shared memory
@@ -525,10 +528,18 @@ int diag_pass(lbm_t h, int i, bool want_u, bool want_aux, int plane_axis, int pl
     // in global memory)
     const double b3 = 3.0 * I.nu0 * I.hist_bins / I.hist_max;  // bin of theta = 3 nu0
     const int lo = b3 >= (double)I.hist_bins ? I.hist_bins : std::max(0, (int)b3 - 1);
-    const int win = std::min(I.hist_bins + 1 - lo, (tma_diag_smem_limit(h->precision) - h->smem) / 4);
-    const int smem_hist = (h->smem + 4 * win + 15) / 16 * 16;
+    const int limit = tma_diag_smem_limit(h->precision);
+    int smem = h->smem;
+    if (want_hist && h->stages > 2 && smem + 4 * (I.hist_bins + 1 - lo) > limit) {
+      // a stage less makes room for all of them: cells beyond the window cost an atomic
+      // in the L2 cache each (128^3 FP16 with a strong strain: 87 us with three stages and a window)
+      lt.stages = h->stages - 1;
+      smem -= h->tile_bytes_max;
+    }
+    const int win = std::min(I.hist_bins + 1 - lo, (limit - smem) / 4);
+    const int smem_hist = (smem + 4 * win + 15) / 16 * 16;
     if (want_hist && win >= kMinHistWindow && tma_prepare(h->precision, smem_hist) == cudaSuccess) {
-      lt.hist_smem = h->smem;
+      lt.hist_smem = smem;
       lt.hist_lo = lo;
       lt.hist_win = win;
       lt.smem_bytes = smem_hist;

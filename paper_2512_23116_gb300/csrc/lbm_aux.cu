@@ -160,11 +160,11 @@ __global__ void k_finish(const double* __restrict__ partials, int ninst, int gri
     const int i = idx / kNP, k = idx - i * kNP;
     const bool lo = k == P_THMIN, hi = k == P_THMAX;
     double r = lo ? DBL_MAX : (hi ? -DBL_MAX : 0.0);
-    for (int b = lane; b < grid; b += 32) {
+#pragma unroll 4
+    for (int b = lane; b < grid; b += 32) {  // unrolled: the loads of four blocks in flight together
       const double* p = partials + ((int64_t)i * grid + b) * kNP;
-      if (p[P_CELLS] == 0.0) continue;  // block saw no cell of instance i
-      const double v = p[k];
-      r = lo ? fmin(r, v) : (hi ? fmax(r, v) : r + v);
+      const double v = p[k], n = p[P_CELLS];
+      if (n != 0.0) r = lo ? fmin(r, v) : (hi ? fmax(r, v) : r + v);  // else the block saw no cell of instance i
     }
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) {
@@ -196,6 +196,7 @@ __global__ void k_sum_cols(const double* __restrict__ p, int rows, int cols, dou
   const int warps = (int)((gridDim.x * blockDim.x) >> 5);
   for (int c = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); c < cols; c += warps) {
     double r = 0.0;
+#pragma unroll 4
     for (int b = lane; b < rows; b += 32) r += p[(int64_t)b * cols + c];
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) r += __shfl_down_sync(0xffffffffu, r, off);

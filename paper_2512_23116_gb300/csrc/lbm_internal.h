@@ -59,7 +59,7 @@ constexpr int kNSum = 16;
 
 // Where a statistics-fused step writes its block partials.
 struct StatsArgs {
-  double* partials;        // [ninst][grid][kNP] (zeroed before the launch)
+  double* partials;        // [ninst][grid][kNP] (zeroed before the launch), or null: no sums
   int32_t grid;            // gridDim.x of the launch
 };
 

@@ -144,7 +144,7 @@ k_step_direct(const InstDesc* __restrict__ insts, int ninst, int64_t chunk_lo, i
     if (t >= w.end) {
       const int ii = ONE ? 0 : find_chunk_instance(insts, ninst, t, cur < 0 ? 0 : cur);
       if (MODE != MODE_STEP) {
-        if (cur >= 0)
+        if (cur >= 0 && sa.partials)
           block_flush(acc, sa.partials + ((int64_t)cur * sa.grid + blockIdx.x) * kNP, blockDim.x, 0);
         acc.reset();
       }
@@ -201,7 +201,7 @@ k_step_direct(const InstDesc* __restrict__ insts, int ninst, int64_t chunk_lo, i
     if (MODE != MODE_STEP) acc.fold_if_full();
   }
   if (MODE != MODE_STEP) {
-    if (cur >= 0)
+    if (cur >= 0 && sa.partials)
       block_flush(acc, sa.partials + ((int64_t)cur * sa.grid + blockIdx.x) * kNP, blockDim.x, 0);
   }
   if (MODE == MODE_DIAG && dout.hist) run.flush(hist_sm, 0, hist_win, hist_gl);

@@ -749,7 +749,7 @@ k_step_tma(const InstDesc* __restrict__ insts, int ninst, int64_t tile_lo, int64
     if (w.ii != cur) {
       // new instance: flush its predecessor's statistics, reload Fz(x) and the
       // per-instance constants
-      if (MODE != MODE_STEP && cur >= 0)
+      if (MODE != MODE_STEP && cur >= 0 && sa.partials)
         block_flush(acc, sa.partials + ((int64_t)cur * sa.grid + blockIdx.x) * kNP, nct, 1);
       acc.reset();
       const InstDesc& d = insts[w.ii];
@@ -807,7 +807,7 @@ k_step_tma(const InstDesc* __restrict__ insts, int ninst, int64_t tile_lo, int64
     __syncwarp();
     if (lane == 0) mbar_arrive(bar_done + 8u * st);
   }
-  if (MODE != MODE_STEP && cur >= 0)
+  if (MODE != MODE_STEP && cur >= 0 && sa.partials)
     block_flush(acc, sa.partials + ((int64_t)cur * sa.grid + blockIdx.x) * kNP, nct, 1);
   if (MODE == MODE_DIAG && dout.hist) run.flush(hist_sm, lo, win, hist_gl);
   if (MODE == MODE_DIAG && dout.hist && hist_sm) {

@@ -39,6 +39,7 @@
 #include "lbm_check.cuh"
 #include "lbm_kernels.h"
 #include "lbm_struct.h"
+#include "lbm_words.cuh"
 
 namespace lbm {
 
@@ -65,27 +66,8 @@ __device__ __forceinline__ void stage4(uint32_t dst, const float* src, bool live
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(n) : "memory");
 }
 
-// A value h + l + m of three FP32 words, |l| <= 2^-24 |h| and m of the order of
-// 2^-48 |h| (a rounded remainder, so the value is good to about 2^-70).
-struct Words {
-  float h, l, m;
-};
-// s + e = a + b exactly (Knuth)
-__device__ __forceinline__ float two_sum(float a, float b, float& e) {
-  const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
-  e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t));
-  return s;
-}
-// Running sums.  The full one keeps every remainder: the odd powers cancel, so
-// their sums feel each term's rounding; the short one drops the remainders of the
-// low words (2^-48 of a term at random), which an even power's sum does not feel.
-__device__ __forceinline__ void add_full(Words& s, const Words& v) {
-  float e, e1, e2;
-  s.h = two_sum(s.h, v.h, e);
-  const float w = two_sum(e, v.l, e1);
-  s.l = two_sum(s.l, w, e2);
-  s.m = __fadd_rn(s.m, __fadd_rn(v.m, __fadd_rn(e1, e2)));
-}
+// s += v without the remainders of the low words (2^-48 of a term at random): enough for the
+// even powers; the odd powers cancel, so their sums feel each term's rounding (add_full).
 __device__ __forceinline__ void add_short(Words& s, const Words& v) {
   float e;
   s.h = two_sum(s.h, v.h, e);
@@ -173,39 +155,13 @@ __device__ __forceinline__ double warp_sums(const PowerSums (&v)[2], int lane) {
   Words a[16];
 #pragma unroll
   for (int i = 0; i < 16; ++i) a[i] = i < 12 ? v[i / 6].s[i % 6] : Words{0.f, 0.f, 0.f};
-#pragma unroll
-  for (int s = 16; s > 0; s >>= 1) {
-    const bool up = (lane & s) != 0;
-#pragma unroll
-    for (int i = 0; i < (s > 1 ? s / 2 : 1); ++i) {
-      Words send = a[i], keep = a[i];
-      if (s > 1) {
-        const Words lo = a[i], hi = a[i + s / 2];
-        send = up ? lo : hi;
-        keep = up ? hi : lo;
-      }
-      const Words o = {__shfl_xor_sync(0xffffffffu, send.h, s), __shfl_xor_sync(0xffffffffu, send.l, s),
-                       __shfl_xor_sync(0xffffffffu, send.m, s)};
-      add_full(keep, o);
-      a[i] = keep;
-    }
-  }
-  return (double)a[0].h + ((double)a[0].l + (double)a[0].m);
+  return to_double(warp_sum16(a, lane));
 }
 __device__ __forceinline__ double warp_sums(const double (&v)[12], int lane) {
   double a[16];
 #pragma unroll
   for (int i = 0; i < 16; ++i) a[i] = i < 12 ? v[i] : 0.0;
-#pragma unroll
-  for (int s = 16; s > 1; s >>= 1) {
-    const bool up = (lane & s) != 0;
-#pragma unroll
-    for (int i = 0; i < s / 2; ++i) {
-      const double send = up ? a[i] : a[i + s / 2], keep = up ? a[i + s / 2] : a[i];
-      a[i] = keep + __shfl_xor_sync(0xffffffffu, send, s);
-    }
-  }
-  return a[0] + __shfl_xor_sync(0xffffffffu, a[0], 1);
+  return warp_sum16(a, lane);
 }
 
 // Sums of one chunk over the run of n cells that starts at p (lane's pencil), FP32.
