@@ -16,6 +16,7 @@
 #include <cstring>
 #include <map>
 #include <string>
+#include <thread>
 #include <vector>
 
 #include "../../include/lbm.h"
@@ -112,6 +113,8 @@ struct lbm_s {
   uint32_t* d_err = nullptr;
   void* d_scratch = nullptr;
   size_t scratch_bytes = 0;
+  char* pin = nullptr;  // page-locked staging of small results
+  size_t pin_bytes = 0;
   double* d_spec = nullptr;
   size_t spec_elems = 0;
   std::map<GraphKey, cudaGraphExec_t> graphs;
@@ -248,6 +251,47 @@ int ensure_scratch(lbm_t h, size_t bytes) {
   CK(h, cudaMalloc(&h->d_scratch, bytes));
   h->scratch_bytes = bytes;
   return LBM_OK;
+}
+
+// Page-locked host memory for results of `bytes`: the copies of a call are enqueued one
+// after the other and waited for once.
+int ensure_pin(lbm_t h, size_t bytes) {
+  if (h->pin_bytes >= bytes) return LBM_OK;
+  if (h->pin) cudaFreeHost(h->pin);
+  h->pin = nullptr;
+  h->pin_bytes = 0;
+  bytes = (bytes + 65535) / 65536 * 65536;
+  CK(h, cudaHostAlloc(reinterpret_cast<void**>(&h->pin), bytes, cudaHostAllocDefault));
+  h->pin_bytes = bytes;
+  return LBM_OK;
+}
+
+// Fault in the pages of an output buffer that is about to be overwritten, by several threads:
+// fresh pages are cleared one by one as they are first written, and a copy that meets
+// them on the way does that on one thread (152 MB: 15 ms, 10 GB/s).
+void touch_pages(void* p, size_t bytes) {
+  constexpr size_t kPage = 4096, kMin = 4 << 20;
+  if (bytes < kMin) return;
+  // plain host memory only: anything else is left to the copy, and to its errors
+  cudaPointerAttributes at{};
+  const bool pending = cudaPeekAtLastError() != cudaSuccess;  // the caller's, left alone
+  if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+    if (!pending) (void)cudaGetLastError();
+    return;
+  }
+  if (at.type != cudaMemoryTypeUnregistered) return;
+  const size_t n = std::min<size_t>({8, std::max(1u, std::thread::hardware_concurrency()), bytes / kMin});
+  auto run = [p, bytes, n](size_t k) {
+    volatile char* c = static_cast<volatile char*>(p);
+    for (size_t i = bytes / n * k, e = k + 1 == n ? bytes : bytes / n * (k + 1); i < e; i += kPage) c[i] = 0;
+  };
+  std::vector<std::thread> pool;
+  try {
+    for (size_t k = 1; k < n; ++k) pool.emplace_back(run, k);
+  } catch (...) {  // no threads to be had: the copy faults the rest in
+  }
+  run(0);
+  for (std::thread& t : pool) t.join();
 }
 
 void clear_graphs(lbm_t h) {
@@ -452,10 +496,14 @@ int run_steps(lbm_t h, int64_t n) {
   return LBM_OK;
 }
 
-int check_err(lbm_t h) {
-  uint32_t e = 0;
-  CK(h, cudaMemcpyAsync(&e, h->d_err, sizeof e, cudaMemcpyDeviceToHost, h->stream));
-  CK(h, cudaStreamSynchronize(h->stream));
+// Enqueue the copy of the device error word to `to` (page-locked).
+int fetch_err(lbm_t h, uint32_t* to) {
+  CK(h, cudaMemcpyAsync(to, h->d_err, sizeof *to, cudaMemcpyDeviceToHost, h->stream));
+  return LBM_OK;
+}
+
+// Report the error word `e` that a synchronised fetch_err has brought.
+int report_err(lbm_t h, uint32_t e) {
   if (kBoundsCheck) {
     const uint32_t b = bounds_word_tma() | bounds_word_direct() | bounds_word_aux() | bounds_word_random() |
                        bounds_word_struct() | bounds_word_spectrum();
@@ -473,6 +521,15 @@ int check_err(lbm_t h) {
     return fail(h, LBM_ERR_UNSTABLE, "non-finite values in the statistics (error word %u)", e);
   }
   return LBM_OK;
+}
+
+int check_err(lbm_t h) {
+  int rc = ensure_pin(h, sizeof(uint32_t));
+  if (rc != LBM_OK) return rc;
+  uint32_t* e = reinterpret_cast<uint32_t*>(h->pin);
+  if ((rc = fetch_err(h, e)) != LBM_OK) return rc;
+  CK(h, cudaStreamSynchronize(h->stream));
+  return report_err(h, *e);
 }
 
 // Read-only pass of the step kernel over instance i: fills the requested
@@ -636,13 +693,16 @@ int max_shell(int nx, int ny, int nz) {
   return (int)(K > r * r + r ? r + 1 : r);
 }
 
-int spectrum_device(lbm_t h, int i, int kmax, double* host_E) {
+// This state's spectrum is at hand.
+bool spectrum_known(lbm_t h, int i, int kmax) {
+  return h->inst[i].spec_version == h->version && h->inst[i].spec_kmax >= kmax;
+}
+
+// Enqueue the spectrum of instance i's velocity (shells 0..kmax) and its copy to the
+// page-locked `host_E`; spectrum_done after a synchronisation.
+int spectrum_enqueue(lbm_t h, int i, int kmax, double* host_E) {
   Inst& I = h->inst[i];
   const lbm_params& p = I.p;
-  if (I.spec_version == h->version && I.spec_kmax >= kmax) {  // this state's spectrum is at hand
-    std::copy(I.spec_E.begin(), I.spec_E.begin() + kmax + 1, host_E);
-    return LBM_OK;
-  }
   if (I.fft_kmax != kmax) {
     cudaError_t pe;
     I.fft_own = plan_fft(p.nx, p.ny, p.nz, kmax, &I.fft, &pe);
@@ -706,11 +766,14 @@ int spectrum_device(lbm_t h, int i, int kmax, double* host_E) {
   const double ncell = (double)p.nx * p.ny * p.nz;
   CK(h, launch_sum_cols(h->d_spec, blocks, kmax + 1, Edev, h->stream, 0.5 / (ncell * ncell)));
   CK(h, cudaMemcpyAsync(host_E, Edev, sizeof(double) * (kmax + 1), cudaMemcpyDeviceToHost, h->stream));
-  CK(h, cudaStreamSynchronize(h->stream));
+  return LBM_OK;
+}
+
+void spectrum_done(lbm_t h, int i, int kmax, const double* host_E) {
+  Inst& I = h->inst[i];
   I.spec_E.assign(host_E, host_E + kmax + 1);
   I.spec_kmax = kmax;
   I.spec_version = h->version;
-  return LBM_OK;
 }
 
 std::vector<int> separations(int n) {
@@ -759,6 +822,7 @@ void release(lbm_t h) {
   cudaFree(h->d_err);
   cudaFree(h->d_scratch);
   cudaFree(h->d_spec);
+  if (h->pin) cudaFreeHost(h->pin);
   if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
   delete h;
 }
@@ -1293,18 +1357,56 @@ LBM_API int lbm_stats(lbm_t h, int32_t inst, int32_t what, lbm_stats_t* out) {
   DevGuard g(h->device);
   Inst& I = h->inst[inst];
   const bool need_u = (what & (LBM_STATS_SPECTRUM | LBM_STATS_STRUCTURE)) != 0;
-  int rc = diag_pass(h, inst, need_u, false, -1, 0, true);
+  const lbm_params& p = I.p;
+  const int kmax = (what & LBM_STATS_SPECTRUM) ? max_shell(p.nx, p.ny, p.nz) : -1;
+  std::vector<int> rs;
+  if (what & LBM_STATS_STRUCTURE) {
+    rs = separations(std::min({p.nx, p.ny, p.nz}));
+    if ((int)rs.size() > LBM_MAX_R) rs.resize(LBM_MAX_R);
+  }
+  const int cols = 6 * (int)rs.size();
+  // page-locked: sums, spectrum, structure functions, histogram, error word
+  const size_t hist_n = (size_t)I.hist_bins + 1;
+  int rc = ensure_pin(h, sizeof(double) * ((size_t)kNP + (kmax + 1) + cols) + sizeof(uint32_t) * (hist_n + 1));
   if (rc != LBM_OK) return rc;
-  std::vector<double> r(kNP);
-  CK(h, cudaMemcpyAsync(r.data(), h->d_results + (size_t)inst * kNP, sizeof(double) * kNP,
-                        cudaMemcpyDeviceToHost, h->stream));
-  std::vector<uint32_t> hist(I.hist_bins + 1);
-  CK(h, cudaMemcpyAsync(hist.data(), I.hist, sizeof(uint32_t) * hist.size(), cudaMemcpyDeviceToHost,
-                        h->stream));
-  rc = check_err(h);
-  if (rc != LBM_OK) return rc;
+  double* r = reinterpret_cast<double*>(h->pin);
+  double* E = r + kNP;
+  double* sp = E + (kmax + 1);
+  uint32_t* hist = reinterpret_cast<uint32_t*>(sp + cols);
+  uint32_t* err = hist + hist_n;
+  // everything is enqueued, then waited for once
+  if ((rc = diag_pass(h, inst, need_u, false, -1, 0, true)) != LBM_OK) return rc;
+  CK(h, cudaMemcpyAsync(r, h->d_results + (size_t)inst * kNP, sizeof(double) * kNP, cudaMemcpyDeviceToHost, h->stream));
+  CK(h, cudaMemcpyAsync(hist, I.hist, sizeof(uint32_t) * hist_n, cudaMemcpyDeviceToHost, h->stream));
+  const bool transform = kmax >= 0 && !spectrum_known(h, inst, kmax);
+  if (transform && (rc = spectrum_enqueue(h, inst, kmax, E)) != LBM_OK) return rc;
+  if (!rs.empty()) {
+    // every separation in one launch into a [blocks][nr x 6] table, one column
+    // sum, one read-back; separations are at most half the smallest extent
+    // (<= 2^10 cells on a lattice of 2^33), which always fits a tile
+    StructPlan plan;
+    cudaError_t pe;
+    if (!plan_struct(p.nx, p.ny, p.nz, rs.data(), (int)rs.size(), false, 4096, &plan, &pe))
+      return fail(h, LBM_ERR_CUDA, "structure functions: %s", cudaGetErrorString(pe));
+    const size_t need = ((size_t)plan.grid + 1) * cols;
+    if (need > h->spec_elems) {
+      if (h->d_spec) cudaFree(h->d_spec);  // waits for the spectrum that still uses it
+      h->d_spec = nullptr;
+      h->spec_elems = 0;
+      CK(h, cudaMalloc(&h->d_spec, need * sizeof(double)));
+      h->spec_elems = need;
+    }
+    CK(h, launch_struct_plan(I.u, plan, false, h->d_spec, h->stream));
+    CK(h, launch_sum_cols(h->d_spec, plan.grid, cols, h->d_spec + (size_t)plan.grid * cols, h->stream));
+    CK(h, cudaMemcpyAsync(sp, h->d_spec + (size_t)plan.grid * cols, sizeof(double) * cols, cudaMemcpyDeviceToHost,
+                          h->stream));
+  }
+  if ((rc = fetch_err(h, err)) != LBM_OK) return rc;
+  CK(h, cudaStreamSynchronize(h->stream));
+  if ((rc = report_err(h, *err)) != LBM_OK) return rc;
+  if (transform) spectrum_done(h, inst, kmax, E);
   std::memset(out, 0, sizeof *out);
-  fill_from_sums(out, r.data(), I, h->t);
+  fill_from_sums(out, r, I, h->t);
   // percentiles: centre of the first bin whose cumulative count reaches p n
   const double pct[4] = {0.05, 0.50, 0.95, 0.99};
   double* dst[4] = {&out->theta_p05, &out->theta_p50, &out->theta_p95, &out->theta_p99};
@@ -1322,12 +1424,8 @@ LBM_API int lbm_stats(lbm_t h, int32_t inst, int32_t what, lbm_stats_t* out) {
   const double nan = std::nan("");
   out->L = out->eps_spec = out->eta = out->lambda = out->u_rms = out->Re_lambda = nan;
   out->u_rms = std::sqrt(2.0 * out->E_k / 3.0);  // Eq. (rms_velocity)
-  const lbm_params& p = I.p;
   if (what & LBM_STATS_SPECTRUM) {
-    const int kmax = max_shell(p.nx, p.ny, p.nz);
-    std::vector<double> E(kmax + 1);
-    rc = spectrum_device(h, inst, kmax, E.data());
-    if (rc != LBM_OK) return rc;
+    const std::vector<double>& E = I.spec_E;
     // Eqs. (integral_length_scale) - (dissipation_rate) with k_s = 2 pi s / nx
     double sE = 0, sEk = 0, sk2E = 0;
     for (int s = 1; s <= kmax; ++s) {
@@ -1343,33 +1441,7 @@ LBM_API int lbm_stats(lbm_t h, int32_t inst, int32_t what, lbm_stats_t* out) {
     out->Re_lambda = out->u_rms * out->lambda / I.nu0;  // Sec. 3.1
   }
   if (what & LBM_STATS_STRUCTURE) {
-    std::vector<int> rs = separations(std::min({p.nx, p.ny, p.nz}));
-    if ((int)rs.size() > LBM_MAX_R) rs.resize(LBM_MAX_R);
-    out->nr = 0;
-    if (rs.empty()) return LBM_OK;
-    // every separation in one launch into a [blocks][nr x 6] table, one column
-    // sum, one read-back; separations are at most half the smallest extent
-    // (<= 2^10 cells on a lattice of 2^33), which always fits a tile
-    const int cols = 6 * (int)rs.size();
-    StructPlan plan;
-    cudaError_t pe;
-    if (!plan_struct(p.nx, p.ny, p.nz, rs.data(), (int)rs.size(), false, 4096, &plan, &pe))
-      return fail(h, LBM_ERR_CUDA, "structure functions: %s", cudaGetErrorString(pe));
-    const size_t need = ((size_t)plan.grid + 1) * cols;
-    if (need > h->spec_elems) {
-      if (h->d_spec) cudaFree(h->d_spec);
-      h->d_spec = nullptr;
-      h->spec_elems = 0;
-      CK(h, cudaMalloc(&h->d_spec, need * sizeof(double)));
-      h->spec_elems = need;
-    }
     out->nr = (int)rs.size();
-    CK(h, launch_struct_plan(I.u, plan, false, h->d_spec, h->stream));
-    CK(h, launch_sum_cols(h->d_spec, plan.grid, cols, h->d_spec + (size_t)plan.grid * cols, h->stream));
-    std::vector<double> sp(cols);
-    CK(h, cudaMemcpyAsync(sp.data(), h->d_spec + (size_t)plan.grid * cols, sizeof(double) * cols,
-                          cudaMemcpyDeviceToHost, h->stream));
-    CK(h, cudaStreamSynchronize(h->stream));
     for (size_t k = 0; k < rs.size(); ++k) {
       out->r[k] = rs[k];
       for (int q = 0; q < 6; ++q) out->Sp[k][q] = sp[6 * k + q] / (3.0 * (double)I.ncell);
@@ -1394,20 +1466,34 @@ LBM_API int lbm_series(lbm_t h, int32_t inst, lbm_record_t* out, int32_t max, in
   if (!count || (max > 0 && !out)) return fail(h, LBM_ERR_INVALID_ARG, "null output");
   DevGuard g(h->device);
   *count = 0;
-  unsigned long long seq = 0;
-  CK(h, cudaMemcpyAsync(&seq, h->d_seq, sizeof seq, cudaMemcpyDeviceToHost, h->stream));
-  int rc = check_err(h);
+  const int ninst = (int)h->inst.size();
+  int rc = ensure_pin(h, sizeof(unsigned long long) + sizeof(uint32_t));
   if (rc != LBM_OK) return rc;
+  unsigned long long* pseq = reinterpret_cast<unsigned long long*>(h->pin);
+  uint32_t* err = reinterpret_cast<uint32_t*>(pseq + 1);
+  CK(h, cudaMemcpyAsync(pseq, h->d_seq, sizeof *pseq, cudaMemcpyDeviceToHost, h->stream));
+  if ((rc = fetch_err(h, err)) != LBM_OK) return rc;
+  CK(h, cudaStreamSynchronize(h->stream));
+  const unsigned long long seq = *pseq;
+  if ((rc = report_err(h, *err)) != LBM_OK) return rc;
   Inst& I = h->inst[inst];
   uint64_t first = I.rec_read;
   if (seq > (unsigned long long)kRingCap && first < seq - kRingCap) first = seq - kRingCap;
-  const int ninst = (int)h->inst.size();
-  std::vector<double> r(kNP);
-  for (uint64_t k = first; k < seq && *count < max; ++k) {
-    CK(h, cudaMemcpy(r.data(), h->d_ring + ((k % kRingCap) * ninst + inst) * kNP,
-                     sizeof(double) * kNP, cudaMemcpyDeviceToHost));
+  // the instance's rows of the ring, at most two runs, in one wait
+  const uint64_t rows = seq > first ? std::min<uint64_t>(seq - first, (uint64_t)std::max(max, 0)) : 0;
+  if ((rc = ensure_pin(h, sizeof(double) * kNP * rows)) != LBM_OK) return rc;
+  double* ring = reinterpret_cast<double*>(h->pin);
+  for (uint64_t k = 0; k < rows;) {
+    const uint64_t slot = (first + k) % kRingCap, run = std::min<uint64_t>(rows - k, kRingCap - slot);
+    CK(h, cudaMemcpy2DAsync(ring + k * kNP, sizeof(double) * kNP, h->d_ring + (slot * ninst + inst) * kNP,
+                            sizeof(double) * kNP * ninst, sizeof(double) * kNP, run, cudaMemcpyDeviceToHost, h->stream));
+    k += run;
+  }
+  if (rows) CK(h, cudaStreamSynchronize(h->stream));
+  for (uint64_t k = first; k < first + rows; ++k) {
+    const double* r = ring + (k - first) * kNP;
     lbm_stats_t s;
-    fill_from_sums(&s, r.data(), I, k < h->rec_steps.size() ? h->rec_steps[k] : -1);
+    fill_from_sums(&s, r, I, k < h->rec_steps.size() ? h->rec_steps[k] : -1);
     lbm_record_t& o = out[*count];
     o.step = s.step;
     o.mass = s.mass;
@@ -1449,14 +1535,28 @@ LBM_API int lbm_spectrum(lbm_t h, int32_t inst, double* E, int32_t kmax) {
   const lbm_params& p = h->inst[inst].p;
   const int smax = max_shell(p.nx, p.ny, p.nz);  // shells beyond hold no mode
   for (int s = smax + 1; s <= kmax; ++s) E[s] = 0.0;
+  Inst& I = h->inst[inst];
+  const int k = std::min(kmax, smax);
   int rc = LBM_OK;
-  if (h->inst[inst].u_version != h->version) {  // the velocity of this state is not at hand
-    rc = diag_pass(h, inst, true, false, -1, 0, false);
-    if (rc != LBM_OK) return rc;
+  if (spectrum_known(h, inst, k)) {
+    if ((rc = check_err(h)) != LBM_OK) return rc;
+  } else {
+    if ((rc = ensure_pin(h, sizeof(double) * (k + 1) + sizeof(uint32_t))) != LBM_OK) return rc;
+    double* host = reinterpret_cast<double*>(h->pin);
+    uint32_t* err = reinterpret_cast<uint32_t*>(host + k + 1);
+    // the velocity of this state may be at hand
+    if (I.u_version != h->version && (rc = diag_pass(h, inst, true, false, -1, 0, false)) != LBM_OK) return rc;
+    if ((rc = spectrum_enqueue(h, inst, k, host)) != LBM_OK) return rc;
+    if ((rc = fetch_err(h, err)) != LBM_OK) return rc;
+    CK(h, cudaStreamSynchronize(h->stream));
+    spectrum_done(h, inst, k, host);
+    if ((rc = report_err(h, *err)) != LBM_OK) {
+      std::copy(I.spec_E.begin(), I.spec_E.begin() + k + 1, E);
+      return rc;
+    }
   }
-  rc = spectrum_device(h, inst, std::min(kmax, smax), E);
-  if (rc != LBM_OK) return rc;
-  return check_err(h);
+  std::copy(I.spec_E.begin(), I.spec_E.begin() + k + 1, E);
+  return LBM_OK;
 }
 
 LBM_API int lbm_histogram(lbm_t h, int32_t inst, uint64_t* counts, int32_t bins) {
@@ -1482,6 +1582,7 @@ LBM_API int lbm_get_populations(lbm_t h, int32_t inst, double* host, int32_t shi
   if (rc != LBM_OK) return rc;
   double* s = static_cast<double*>(h->d_scratch);
   const bool odd = (h->t & 1) != 0;
+  touch_pages(host, sizeof(double) * 19 * (size_t)I.ncell);
   for (int a = 0; a < 19; ++a)
     for (int64_t c0 = 0; c0 < I.ncell; c0 += chunk) {
       const int64_t n = std::min(chunk, I.ncell - c0);
@@ -1540,12 +1641,17 @@ LBM_API int lbm_get_fields(lbm_t h, int32_t inst, double* drho, double* u, doubl
   Inst& I = h->inst[inst];
   int rc = diag_pass(h, inst, u != nullptr, drho || snorm || theta, -1, 0, false);
   if (rc != LBM_OK) return rc;
-  std::vector<float> buf;
+  // widened on the device, copied straight into the caller's array
+  const int64_t chunk = std::min<int64_t>(3 * I.ncell, kChunkCells);
+  if ((rc = ensure_scratch(h, sizeof(double) * (size_t)chunk)) != LBM_OK) return rc;
   auto fetch = [&](const float* src, double* dst, int64_t n) -> int {
-    buf.resize((size_t)n);
-    CK(h, cudaMemcpyAsync(buf.data(), src, sizeof(float) * n, cudaMemcpyDeviceToHost, h->stream));
-    CK(h, cudaStreamSynchronize(h->stream));
-    for (int64_t k = 0; k < n; ++k) dst[k] = buf[k];
+    touch_pages(dst, sizeof(double) * (size_t)n);
+    double* s = static_cast<double*>(h->d_scratch);
+    for (int64_t c0 = 0; c0 < n; c0 += chunk) {
+      const int64_t m = std::min(chunk, n - c0);
+      CK(h, launch_widen(src + c0, m, s, h->stream));
+      CK(h, cudaMemcpyAsync(dst + c0, s, sizeof(double) * m, cudaMemcpyDeviceToHost, h->stream));
+    }
     return LBM_OK;
   };
   if (u && (rc = fetch(I.u, u, 3 * I.ncell)) != LBM_OK) return rc;
@@ -1572,11 +1678,18 @@ LBM_API int lbm_get_theta_slice(lbm_t h, int32_t inst, int32_t axis, int32_t ind
   int rc = diag_pass(h, inst, false, false, axis, index, false);
   if (rc != LBM_OK) return rc;
   const size_t n = axis == 0 ? (size_t)p.nz * p.ny : (axis == 1 ? (size_t)p.nz * p.nx : (size_t)p.ny * p.nx);
-  std::vector<float> buf(n);
-  CK(h, cudaMemcpyAsync(buf.data(), I.plane, sizeof(float) * n, cudaMemcpyDeviceToHost, h->stream));
-  CK(h, cudaStreamSynchronize(h->stream));
-  for (size_t k = 0; k < n; ++k) host[k] = buf[k];
-  return check_err(h);
+  const size_t chunk = std::min(n, (size_t)kChunkCells);
+  if ((rc = ensure_pin(h, sizeof(float) * (chunk + 1))) != LBM_OK) return rc;
+  float* buf = reinterpret_cast<float*>(h->pin);
+  uint32_t* err = reinterpret_cast<uint32_t*>(buf + chunk);
+  if ((rc = fetch_err(h, err)) != LBM_OK) return rc;
+  for (size_t c0 = 0; c0 < n; c0 += chunk) {
+    const size_t m = std::min(chunk, n - c0);
+    CK(h, cudaMemcpyAsync(buf, I.plane + c0, sizeof(float) * m, cudaMemcpyDeviceToHost, h->stream));
+    CK(h, cudaStreamSynchronize(h->stream));
+    for (size_t k = 0; k < m; ++k) host[c0 + k] = buf[k];
+  }
+  return report_err(h, *err);
 }
 
 LBM_API int lbm_device_ptr(lbm_t h, int32_t inst, void** ptr, size_t* bytes, int32_t* nxp) {

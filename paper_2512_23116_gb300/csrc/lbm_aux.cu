@@ -108,6 +108,11 @@ __global__ void k_set_pop(InstDesc d, bool odd, int a, const double* __restrict_
   }
 }
 
+__global__ void k_widen(const float* __restrict__ in, int64_t n, double* __restrict__ out) {
+  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x)
+    out[k] = (double)in[k];
+}
+
 // sa, sb: dense [nz][ny][nxp] copies of slots a and opp(a) taken at the old parity.
 template <typename T>
 __global__ void k_relayout(InstDesc d, bool from_odd, int a, const T* __restrict__ sa,
@@ -263,6 +268,11 @@ cudaError_t launch_set_pop(const InstDesc& d, int precision, bool odd, int a, co
     case 2: return launch_kernel(k_set_pop<__nv_bfloat16>, g, kAuxThreads, 0, st, d, odd, a, in, shifted, c0, n);
   }
   return cudaErrorInvalidValue;
+}
+
+cudaError_t launch_widen(const float* in, int64_t n, double* out, cudaStream_t st) {
+  if (n <= 0) return cudaSuccess;
+  return launch_kernel(k_widen, grid_for(n), kAuxThreads, 0, st, in, n, out);
 }
 
 cudaError_t launch_relayout_pair(const InstDesc& d, int precision, bool from_odd, int a,

@@ -119,6 +119,8 @@ cudaError_t launch_get_pop(const InstDesc& d, int precision, bool odd, int a, do
                            int shifted, int64_t c0, int64_t n, cudaStream_t st);
 cudaError_t launch_set_pop(const InstDesc& d, int precision, bool odd, int a, const double* in,
                            int shifted, int64_t c0, int64_t n, cudaStream_t st);
+// out[k] = in[k], k < n.
+cudaError_t launch_widen(const float* in, int64_t n, double* out, cudaStream_t st);
 // Re-lay out the pair (a, opp a) from parity `from_odd` to the other parity
 // using a scratch buffer of 2 * nz * ny * nxp storage elements.
 cudaError_t launch_relayout_pair(const InstDesc& d, int precision, bool from_odd, int a,
