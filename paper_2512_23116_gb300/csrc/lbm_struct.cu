@@ -15,10 +15,11 @@
 // Two accuracies share that skeleton:
 //  - k_struct_tiles<false>, for lbm_stats: FP32 increments and powers as the
 //    FP32 velocity allows, summed in FP32 over at most kRunMax cells of a lane
-//    and the lanes of its warp, then in FP64.  Bound by issue: 10 instructions an
-//    increment (9 FP32 operations and a load), 73 % of the issue rate at 400^3.
-//    All separations of a call: 100^3 (11 of them) 102 -> 23 us, 400^3 (15)
-//    3.11 -> 1.34 ms, 512^3 (16) 8.5 -> 2.75 ms.
+//    and the lanes of its warp, then in FP64.  Two separations share a register
+//    pair (f32x2 operations), which halves the issue slots of the 9 operations an increment
+//    takes and leaves the FP32 pipe as the bound (0.74 ms of it at 400^3).
+//    All separations of a call: 100^3 (11 of them) 102 -> 20 us, 400^3 (15)
+//    3.11 -> 1.27 ms, 512^3 (16) 8.5 -> 2.58 ms; without the pairs 23 us, 1.34 and 2.75 ms.
 //  - k_struct_tiles<true>, for lbm_structure_functions_noalloc: the FP64 sums of
 //    the exact increments.  This part executes 2 FP64 operations per clock and
 //    SM against 128 in FP32, so increments, powers and running sums are kept as
@@ -164,25 +165,61 @@ __device__ __forceinline__ double warp_sums(const double (&v)[12], int lane) {
   return warp_sum16(a, lane);
 }
 
-// Sums of one chunk over the run of n cells that starts at p (lane's pencil), FP32.
+// Two FP32 values in one 64-bit register, operated on together (add / mul / fma.f32x2:
+// one issue slot for two operations, each rounded as the scalar one).
+using Pair = unsigned long long;
+__device__ __forceinline__ Pair pack2(float x, float y) {
+  Pair r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+  return r;
+}
+__device__ __forceinline__ void unpack2(Pair a, float& x, float& y) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(a));
+}
+__device__ __forceinline__ Pair add2(Pair a, Pair b) {
+  Pair r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ Pair mul2(Pair a, Pair b) {
+  Pair r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ Pair fma2(Pair a, Pair b, Pair c) {
+  Pair r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+
+// Sums of one chunk over the run of n cells that starts at p (lane's pencil), FP32, two
+// separations to a register pair.
 __device__ __forceinline__ void run_f32(const float* p, const int (&off)[4], int n, float (&t)[24]) {
+  Pair s[2][6];
 #pragma unroll
-  for (int i = 0; i < 24; ++i) t[i] = 0.f;
-#pragma unroll 4
+  for (int j = 0; j < 2; ++j)
+#pragma unroll
+    for (int k = 0; k < 6; ++k) s[j][k] = 0ull;
+#pragma unroll 8
   for (int i = 0; i < n; ++i, p += kPitch) {
-    const float own = p[0];
+    const float own = -p[0];
+    const Pair own2 = pack2(own, own);
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const float d = p[off[j]] - own;
-      const float q = d * d, c = q * d;
-      t[6 * j] += d;
-      t[6 * j + 1] += q;
-      t[6 * j + 2] = fmaf(q, d, t[6 * j + 2]);
-      t[6 * j + 3] = fmaf(q, q, t[6 * j + 3]);
-      t[6 * j + 4] = fmaf(c, q, t[6 * j + 4]);
-      t[6 * j + 5] = fmaf(c, c, t[6 * j + 5]);
+    for (int j = 0; j < 2; ++j) {
+      const Pair d = add2(pack2(p[off[2 * j]], p[off[2 * j + 1]]), own2);
+      const Pair q = mul2(d, d), c = mul2(q, d);
+      s[j][0] = add2(s[j][0], d);
+      s[j][1] = add2(s[j][1], q);
+      s[j][2] = fma2(q, d, s[j][2]);
+      s[j][3] = fma2(q, q, s[j][3]);
+      s[j][4] = fma2(c, q, s[j][4]);
+      s[j][5] = fma2(c, c, s[j][5]);
     }
   }
+#pragma unroll
+  for (int j = 0; j < 2; ++j)
+#pragma unroll
+    for (int k = 0; k < 6; ++k) unpack2(s[j][k], t[12 * j + k], t[12 * j + 6 + k]);
 }
 
 // The same in three-word arithmetic, increments times `scale` (a power of two).
