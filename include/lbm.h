@@ -74,7 +74,7 @@ extern "C" {
 #define LBM_INIT_VELOCITY 3     /* u from the caller, drho = 0 */
 
 /* Which quantities lbm_stats computes beyond the fused domain sums. */
-#define LBM_STATS_SPECTRUM 1    /* derived scales from E(k) (needs cuFFT) */
+#define LBM_STATS_SPECTRUM 1    /* derived scales from E(k) */
 #define LBM_STATS_STRUCTURE 2   /* S_p(r), p = 1..6, and F4(r) */
 
 #define LBM_MAX_R 24
@@ -289,7 +289,8 @@ int lbm_energy_balance(const lbm_record_t* rec, int32_t n, double* residual, int
 
 /* Energy spectrum E(s), s = 0..kmax, of Eq. (integral_length_scale) with
  * |u_hat|^2, u_hat = N^-3 sum_x u exp(-2 pi i k.x/N), integer shells
- * s - 1/2 <= |k| < s + 1/2 (cuFFT R2C in FP32, shell sums in FP64).  E points
+ * s - 1/2 <= |k| < s + 1/2 (FP32 transform, shell sums in FP64; extents with prime
+ * factors above 13 by cuFFT).  E points
  * to kmax + 1 doubles of host memory.  Synchronous.  Errors: INVALID_ARG
  * (kmax < 0), CUDA (cuFFT failures included). */
 int lbm_spectrum(lbm_t h, int32_t inst, double* E, int32_t kmax);

@@ -37,6 +37,7 @@ constexpr int kMinHistWindow = 256;  // fewer histogram bins than this in shared
 constexpr int64_t kChunkCells = 4 << 20;
 constexpr size_t kDirectBytes = 24 << 20;     // populations up to this size: direct kernel, no others timed
 constexpr size_t kDirectMaxBytes = 40 << 20;  // and up to this size (FP32): the direct kernel among others
+constexpr size_t kPinBytes = 256 << 10;       // page-locked staging of small results, at least
 constexpr size_t kFftBatchBytes = 192 << 20;  // three half spectra (256^3) transformed together
 constexpr double kPi = 3.14159265358979323846;
 
@@ -795,6 +796,9 @@ int alloc_common(lbm_t h) {
   CK(h, cudaMalloc(&h->d_ring, sizeof(double) * kNP * h->inst.size() * kRingCap));
   CK(h, cudaMalloc(&h->d_seq, 2 * sizeof(unsigned long long)));
   CK(h, cudaMalloc(&h->d_err, sizeof(uint32_t)));
+  // here and not in the first call that needs it: page-locking waits for the device
+  const int rc = ensure_pin(h, kPinBytes);
+  if (rc != LBM_OK) return rc;
   CK(h, cudaMemsetAsync(h->d_seq, 0, 2 * sizeof(unsigned long long), h->stream));
   CK(h, cudaMemsetAsync(h->d_err, 0, sizeof(uint32_t), h->stream));
   return LBM_OK;
@@ -1678,7 +1682,7 @@ LBM_API int lbm_get_theta_slice(lbm_t h, int32_t inst, int32_t axis, int32_t ind
   int rc = diag_pass(h, inst, false, false, axis, index, false);
   if (rc != LBM_OK) return rc;
   const size_t n = axis == 0 ? (size_t)p.nz * p.ny : (axis == 1 ? (size_t)p.nz * p.nx : (size_t)p.ny * p.nx);
-  const size_t chunk = std::min(n, (size_t)kChunkCells);
+  const size_t chunk = std::min(n, kPinBytes / sizeof(float) - 1);  // larger planes in pieces
   if ((rc = ensure_pin(h, sizeof(float) * (chunk + 1))) != LBM_OK) return rc;
   float* buf = reinterpret_cast<float*>(h->pin);
   uint32_t* err = reinterpret_cast<uint32_t*>(buf + chunk);
