@@ -141,12 +141,24 @@ __device__ __forceinline__ void named_sync(int bar_id, int nthreads) {
 // warp with a shuffle tree per value: 19 us a statistics step of 32^3 and 28 of 64^3,
 // now 6 and 10.5; 100^3 38 -> 25): the
 // 16 sums are reduced together, each step halving the values a lane holds, the FP32
-// part in three FP32 words (nothing lost against FP64) and the FP64 totals only
-// where some lane has folded into them; extrema and counts need no FP64.
+// part in three FP32 words and the FP64 totals only where some lane has folded into
+// them; extrema and counts need no FP64.  The words hold what FP64 would while the
+// lanes' sums stay clear of the ends of the FP32 range: 32 sums below 2^115 cannot
+// overflow, and above 2^-64 what the low words lose by flushing (2^-126 a term) is below
+// FP64's rounding.  A warp with a sum outside (infinities and NaN included) folds
+// it into its FP64 totals first.
+constexpr uint32_t kWordsLo = (127u - 64u) << 23, kWordsHi = (127u + 115u) << 23;  // 2^-64, 2^115
 static __device__ __forceinline__ void block_flush(Acc& acc, double* __restrict__ dst, int nthreads,
                                          int bar_id) {
   __shared__ double red[32][kNP];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  bool outside = false;
+#pragma unroll
+  for (int k = 0; k < kNSum; ++k) {
+    const uint32_t m = __float_as_uint(acc.t[k]) & 0x7fffffffu;
+    outside |= m != 0u && m - kWordsLo > kWordsHi - kWordsLo;
+  }
+  if (__any_sync(0xffffffffu, outside)) acc.fold();
   Words t[kNSum];
 #pragma unroll
   for (int k = 0; k < kNSum; ++k) t[k] = Words{acc.t[k], 0.f, 0.f};
