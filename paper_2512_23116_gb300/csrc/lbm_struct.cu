@@ -24,14 +24,14 @@
 //    the exact increments.  This part executes 2 FP64 operations per clock and
 //    SM against 128 in FP32, so increments, powers and running sums are kept as
 //    unevaluated sums of FP32 words (Dekker 1971; Knuth's two-sum, products with
-//    an FMA for the remainder).  Against quadruple-precision sums it is off by 1-2e-16
-//    of S_2, S_4, S_6 and 1-7e-18 of <|d|^3>, <|d|^5> on lattices of 1.0e5 to 1.4e6 cells,
-//    where the FP64 loop left 3-7e-16 and 1e-18-2e-17.  Each tile scales its increments
-//    by a power of two so that neither the sixth power nor its low words leave the
-//    FP32 range; a tile whose values do not allow that (infinities, NaN, extreme
-//    exponents) is summed in FP64.  Bound by issue: ~180 FP32 operations an
-//    increment.  12 separations at 160^3: 4.43 ms (one FP64 pass over global memory
-//    per separation, at the FP64 rate) -> 0.94 ms.
+//    an FMA for the remainder).  Against quadruple-precision sums it is off by at most
+//    6e-16 of <|d|^p> for every p, on random, Taylor-Green, sinusoidal and ramp fields of
+//    7e4 to 1e6 cells (2e-16 typically), where the FP64 loop left 0.3-1.2e-14.  Each tile
+//    scales its increments by a power of two so that neither the sixth power nor its low
+//    words leave the FP32 range; a tile whose values do not allow that (infinities, NaN,
+//    extreme exponents) is summed in FP64.  Bound by issue: ~215 FP32 operations an
+//    increment.  12 separations at 160^3: 4.50 ms (one FP64 pass over global memory
+//    per separation, at the FP64 rate) -> 1.14 ms.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -67,17 +67,10 @@ __device__ __forceinline__ void stage4(uint32_t dst, const float* src, bool live
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(n) : "memory");
 }
 
-// s += v without the remainders of the low words (2^-48 of a term at random): enough for the
-// even powers; the odd powers cancel, so their sums feel each term's rounding (add_full).
-__device__ __forceinline__ void add_short(Words& s, const Words& v) {
-  float e;
-  s.h = two_sum(s.h, v.h, e);
-  s.l = __fadd_rn(s.l, __fadd_rn(e, v.l));
-  s.m = __fadd_rn(s.m, v.m);
-}
-// a b to three words, every term down to second order; short: only those second-order
-// terms that do not average out (l l and h m: a low word rounds them away
-// always in the same direction, 2e-15 of a sum of even powers).
+// a b to three words, every term down to second order.  None may be left out, and no
+// remainder of a running sum: a low word rounds what is dropped at 2^-48 of a term, and
+// fields whose pencils repeat do so alike in every lane and run (sums of d^4 and d^6
+// were off by 1-2e-14 of a sinusoid or a ramp, where FP64 loops leave 0.5-1e-14).
 __device__ __forceinline__ Words mul_full(const Words& a, const Words& b) {
   Words c;
   c.h = __fmul_rn(a.h, b.h);
@@ -90,7 +83,7 @@ __device__ __forceinline__ Words mul_full(const Words& a, const Words& b) {
   c.m = __fmaf_rn(a.l, b.l, __fmaf_rn(a.h, b.m, __fmaf_rn(a.m, b.h, __fadd_rn(__fadd_rn(r1, r2), __fadd_rn(y1, y2)))));
   return c;
 }
-__device__ __forceinline__ Words sqr_full(const Words& a) {  // a.m = 0
+__device__ __forceinline__ Words sqr_two(const Words& a) {  // a.m = 0
   Words c;
   c.h = __fmul_rn(a.h, a.h);
   const float t = __fmaf_rn(a.h, a.h, -c.h), a2 = __fadd_rn(a.h, a.h);
@@ -100,12 +93,9 @@ __device__ __forceinline__ Words sqr_full(const Words& a) {  // a.m = 0
   c.m = __fmaf_rn(a.l, a.l, __fadd_rn(r, y));
   return c;
 }
-__device__ __forceinline__ Words sqr_short(const Words& a) {
-  Words c;
-  c.h = __fmul_rn(a.h, a.h);
-  const float a2 = __fadd_rn(a.h, a.h);
-  c.l = __fmaf_rn(a2, a.l, __fmaf_rn(a.h, a.h, -c.h));
-  c.m = __fmaf_rn(a.l, a.l, __fmul_rn(a2, a.m));
+__device__ __forceinline__ Words sqr_full(const Words& a) {
+  Words c = sqr_two(a);
+  c.m = __fmaf_rn(__fadd_rn(a.h, a.h), a.m, c.m);
   return c;
 }
 
@@ -121,13 +111,13 @@ struct PowerSums {
     float e;
     const float r = two_sum(a, -b, e);
     const Words d = {__fmul_rn(r, scale), __fmul_rn(e, scale), 0.f};
-    const Words q = sqr_full(d), c = mul_full(q, d);
+    const Words q = sqr_two(d), c = mul_full(q, d);
     add_full(s[0], d);
-    add_full(s[1], q);  // its low words have few bits, whose sum would round with a bias
+    add_full(s[1], q);
     add_full(s[2], c);
-    add_short(s[3], sqr_short(q));
+    add_full(s[3], sqr_full(q));
     add_full(s[4], mul_full(c, q));
-    add_short(s[5], sqr_short(c));
+    add_full(s[5], sqr_full(c));
   }
 };
 
