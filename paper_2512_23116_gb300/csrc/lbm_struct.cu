@@ -243,14 +243,21 @@ __device__ __noinline__ void run_f64(const float* p, int off0, int off1, int n, 
 // stays below 2^19, its sixth power below 2^114 and a run's sum below 2^120; its
 // low parts keep all their bits down to increments 2^-20 of that largest one,
 // whose share of a sum is below the FP64 rounding.  INT_MIN when the
-// values do not allow it.
+// values do not allow it.  adj is zero only when every pencil is constant bit by bit
+// (cells_differ): differences below the normal range flush to zero in FP32, not in FP64.
 __device__ __forceinline__ int tile_exponent(float adj, float top) {
-  if (adj == 0.f && top < 1e30f) return 0;  // constant pencils: every increment is zero
+  if (adj == 0.f && top < 1e30f) return 0;  // every increment is zero
   if (!(adj >= 0x1p-60f && adj < 0x1p60f && top < 0x1p60f)) return INT_MIN;
   const int e = (int)(__float_as_uint(adj) >> 23) - 127;
   const int k = 7 - e;
   const int et = (int)(__float_as_uint(top) >> 23) - 127;
   return et + k < 120 ? k : INT_MIN;
+}
+
+// The values differ (zeros of either sign are alike).
+__device__ __forceinline__ bool cells_differ(float a, float b) {
+  const uint32_t x = __float_as_uint(a), y = __float_as_uint(b);
+  return x != y && ((x | y) << 1) != 0u;
 }
 
 // Tiles of the three axes in one numbering; a block takes tiles b, b + grid, ...
@@ -303,14 +310,19 @@ k_struct_tiles(const float* __restrict__ u, StructPlan pl, double* __restrict__ 
     int kexp = 0;
     if (EXACT) {
       float adj = 0.f, top = 0.f;
-      bool odd = false;  // NaN: fmaxf would drop it
+      bool odd = false, moved = false;  // odd: NaN, which fmaxf would drop
       for (int i = warp; i < rows; i += nwarps) {
         const float v = tile[i * kPitch + lane];
         top = fmaxf(top, fabsf(v));
         odd |= !(fabsf(v) < 0x1p60f);
-        if (i + 1 < rows) adj = fmaxf(adj, fabsf(tile[(i + 1) * kPitch + lane] - v));
+        if (i + 1 < rows) {
+          const float w = tile[(i + 1) * kPitch + lane];
+          adj = fmaxf(adj, fabsf(w - v));
+          moved |= cells_differ(v, w);
+        }
       }
       if (odd) top = 0x1p100f;
+      if (moved) adj = fmaxf(adj, 0x1p-126f);
 #pragma unroll
       for (int off = 16; off > 0; off >>= 1) {
         adj = fmaxf(adj, __shfl_xor_sync(0xffffffffu, adj, off));
