@@ -50,11 +50,6 @@ constexpr int kCols = 32;       // pencils of a tile: one per lane
 constexpr int kPitch = 33;      // values between consecutive cells of a pencil
 constexpr int kRunMax = 64;     // cells a lane sums before the warp reduces
 constexpr int kWarpsMax = 8;
-// Lattices below this many cells are summed in FP64 terms: on 7,680 cells the
-// roundings of the three-word even powers left 1.7-2.9e-16 of S_2, S_4, S_6 where
-// FP64 left 0.7-1.5e-16; from 96,000 cells on they leave less (1e-16 against
-// 4-5e-16).
-constexpr int64_t kWordsCells = 1 << 16;
 constexpr int kSmemMax = 225 * 1024;  // dynamic shared memory of a block, beside the few static words
 
 // Separations of one pass over a tile: its sums stay in registers (24 FP32 sums
@@ -337,7 +332,7 @@ k_struct_tiles(const float* __restrict__ u, StructPlan pl, double* __restrict__ 
         adj = fmaxf(adj, s_adj[w]);
         top = fmaxf(top, s_top[w]);
       }
-      kexp = pl.fp64 ? INT_MIN : tile_exponent(adj, top);
+      kexp = tile_exponent(adj, top);
     }
     const int q = (len + nwarps - 1) / nwarps;
     const int n = max(0, min(q, len - warp * q));
@@ -493,7 +488,6 @@ bool plan_struct(int nx, int ny, int nz, const int* r, int nr, bool exact, int m
   }
   pl.rows_max += pl.rows_max & 1;  // the FP64 sums behind the tile start on 8 bytes
   pl.tiles = tiles;
-  pl.fp64 = pl.ncell < kWordsCells;
   pl.threads = 32 * warps;
   const size_t smem = (size_t)pl.rows_max * kPitch * 4 + warps * sums;
   *err = cudaSuccess;

@@ -26,7 +26,6 @@ struct StructPlan {
   int nx, nr;
   int rows_max;                 // longest tile: segment plus halo
   int r[3][kMaxStructSeps];     // separations wrapped to each extent
-  int fp64;                     // exact sums by FP64 terms
   int grid, threads, smem;
 };
 
