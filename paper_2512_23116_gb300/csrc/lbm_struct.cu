@@ -49,6 +49,7 @@ namespace {
 constexpr int kCols = 32;       // pencils of a tile: one per lane
 constexpr int kPitch = 33;      // values between consecutive cells of a pencil
 constexpr int kRunMax = 64;     // cells a lane sums before the warp reduces
+constexpr int kRunMin = 4;      // fewer are not worth the reduction
 constexpr int kWarpsMax = 8;
 constexpr int kSmemMax = 225 * 1024;  // dynamic shared memory of a block, beside the few static words
 
@@ -431,13 +432,11 @@ __global__ void k_struct(const float* __restrict__ u, int nx, int ny, int nz, in
 }
 
 template <bool EXACT>
-cudaError_t finish_plan(StructPlan& pl, int max_blocks) {
+cudaError_t finish_plan(StructPlan& pl, int max_blocks, int sms) {
   cudaError_t e = cudaFuncSetAttribute(k_struct_tiles<EXACT>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
-  int per_sm = 0, dev = 0, sms = 0;
+  int per_sm = 0;
   if (e == cudaSuccess)
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_struct_tiles<EXACT>, pl.threads, pl.smem);
-  if (e == cudaSuccess) e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e == cudaSuccess && per_sm < 1) e = cudaErrorInvalidConfiguration;
   if (e == cudaSuccess)
     pl.grid = (int)std::max<int64_t>(1, std::min<int64_t>({pl.tiles, (int64_t)per_sm * sms, (int64_t)max_blocks}));
@@ -473,28 +472,42 @@ bool plan_struct(int nx, int ny, int nz, const int* r, int nr, bool exact, int m
   // at most kRunMax cells per warp.
   const int short_rows = std::min(longest, 4 * kRunMax) + halo;
   const int warps = longest <= 4 * kRunMax && (size_t)short_rows * kPitch * 4 + 4 * sums <= 36 * 1024 ? 4 : kWarpsMax;
-  int64_t tiles = 0;
-  for (int a = 0; a < 3; ++a) {
-    StructAxis& ax = pl.ax[a];
-    ax.n = n[a];
-    ax.stride = a == 0 ? 1 : (a == 1 ? (int64_t)nx : pl.plane);
-    ax.pencils = pl.ncell / n[a];
-    ax.segs = (n[a] + warps * kRunMax - 1) / (warps * kRunMax);
-    ax.len = (n[a] + ax.segs - 1) / ax.segs;
-    ax.segs = (n[a] + ax.len - 1) / ax.len;
-    ax.first = tiles;
-    tiles += (ax.pencils + kCols - 1) / kCols * ax.segs;
-    pl.rows_max = std::max(pl.rows_max, ax.len + ax.halo);
-  }
-  pl.rows_max += pl.rows_max & 1;  // the FP64 sums behind the tile start on 8 bytes
-  pl.tiles = tiles;
+  auto cut = [&](int64_t least) {  // into `least` tiles an axis or more, runs of kRunMin cells or more
+    int64_t tiles = 0;
+    pl.rows_max = 0;
+    for (int a = 0; a < 3; ++a) {
+      StructAxis& ax = pl.ax[a];
+      ax.n = n[a];
+      ax.stride = a == 0 ? 1 : (a == 1 ? (int64_t)nx : pl.plane);
+      ax.pencils = pl.ncell / n[a];
+      const int64_t cols = (ax.pencils + kCols - 1) / kCols;
+      ax.segs = std::max((n[a] + warps * kRunMax - 1) / (warps * kRunMax),
+                         (int)std::min<int64_t>(least / cols, n[a] / (warps * kRunMin)));
+      ax.len = (n[a] + ax.segs - 1) / ax.segs;
+      ax.segs = (n[a] + ax.len - 1) / ax.len;
+      ax.first = tiles;
+      tiles += cols * ax.segs;
+      pl.rows_max = std::max(pl.rows_max, ax.len + ax.halo);
+    }
+    pl.rows_max += pl.rows_max & 1;  // the FP64 sums behind the tile start on 8 bytes
+    pl.tiles = tiles;
+    return (size_t)pl.rows_max * kPitch * 4 + warps * sums;
+  };
+  size_t smem = cut(0);
   pl.threads = 32 * warps;
-  const size_t smem = (size_t)pl.rows_max * kPitch * 4 + warps * sums;
   *err = cudaSuccess;
   // an increment spans at most 2^11 cells (tile_exponent)
   if (smem > (size_t)kSmemMax || pl.rows_max > 2048) return false;
+  int dev = 0, sms = 0;
+  *err = cudaGetDevice(&dev);
+  if (*err == cudaSuccess) *err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (*err != cudaSuccess) return false;
+  // Exact sums: a long box has few pencils along its length, whose tiles of 8 x 64 cells
+  // would keep a few SMs busy for long (2000 x 2 x 2, 24 separations: 456 us in 4 tiles).
+  // Shorter segments give every SM one.
+  if (exact) smem = cut(sms);
   pl.smem = (int)smem;
-  *err = exact ? finish_plan<true>(pl, max_blocks) : finish_plan<false>(pl, max_blocks);
+  *err = exact ? finish_plan<true>(pl, max_blocks, sms) : finish_plan<false>(pl, max_blocks, sms);
   *out = pl;
   return *err == cudaSuccess;
 }

@@ -1,0 +1,40 @@
+"""Exact structure functions of long boxes, whose pencils are cut into short segments so
+that every SM has a tile: the sums, and that a long box takes about as long as a cube."""
+import numpy as np
+import pytest
+
+from test_gpu_struct import _noalloc, _sums
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("shape", [(2, 2, 2000), (2000, 2, 2), (2, 1999, 3), (8, 8, 3000), (1, 1, 1000)])
+@pytest.mark.parametrize("seps", [[1], [1, 2, 31, 33, 500], [999]])
+def test_long_boxes(gpu_lib, shape, seps):
+    u = np.random.default_rng(8).normal(scale=0.05, size=(3, *shape)).astype(np.float32)
+    want, mag = _sums(u, seps)
+    assert np.all(np.abs(_noalloc(gpu_lib, u, seps) - want) <= 1e-14 * mag)
+
+
+def _device_time(lbm, shape, seps):
+    import torch
+    u = torch.randn((3, *shape), generator=torch.Generator("cuda").manual_seed(1), device="cuda") * 0.05
+    sp = torch.empty(len(seps), 6, dtype=torch.float64, device="cuda")
+    st = torch.cuda.current_stream()
+    times = []
+    for _ in range(7):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        for _ in range(10):
+            lbm.lbm_structure_functions_noalloc(u, seps, sp, stream=st)
+        b.record()
+        torch.cuda.synchronize()
+        times.append(a.elapsed_time(b))
+    return sorted(times)[3]
+
+
+def test_a_long_box_takes_no_longer_than_its_cells_need(gpu_lib):
+    """8,000 cells either way; 4 tiles on 4 SMs took 10 and more times the cube's time.  The
+    long box stages more halo: 3 times is allowed."""
+    seps = list(range(1, 25))
+    assert _device_time(gpu_lib, (2, 2, 2000), seps) <= 3 * _device_time(gpu_lib, (20, 20, 20), seps)
