@@ -13,20 +13,24 @@
 // the shifted loads (9 % of the DRAM peak at 256^3).
 //
 // Two accuracies share that skeleton:
-//  - k_struct_tiles<false>, for lbm_stats: FP32 increments and powers as the
-//    FP32 velocity allows, summed in FP32 over at most kRunMax cells of a lane
-//    and the lanes of its warp, then in FP64.  Two separations share a register
-//    pair (f32x2 operations), which halves the issue slots of the 9 operations an increment
-//    takes and leaves the FP32 pipe as the bound (0.74 ms of it at 400^3).
-//    All separations of a call: 100^3 (11 of them) 102 -> 20 us, 400^3 (15)
-//    3.11 -> 1.27 ms, 512^3 (16) 8.5 -> 2.58 ms; without the pairs 23 us, 1.34 and 2.75 ms.
-//  - k_struct_tiles<true>, for lbm_structure_functions_noalloc: the FP64 sums of
+//  - k_struct_tiles<SUMS_4> and <SUMS_1>, for lbm_stats: FP32 increments and powers as
+//    the FP32 velocity allows.  Plain FP32 sums span 4 cells; over a lane's run those of
+//    the odd powers, and over the warp all of them, are kept in two words, then added in
+//    FP64.  Lattices up to kSmallCells have few cells for roundings to average over, and
+//    time to spare: no plain sums at all.  Two separations share a register pair (f32x2
+//    operations).  Against FP64 sums of random solenoidal fields S_1 to S_6 are off by
+//    2e-11 to 6e-10 of <|d|^p> at 100^3 and 7e-12 to 2e-9 at 404^3; plain sums of 64 cells
+//    and the warp left S_1, S_3 and S_5 3-18 times that.  Bound by the FP32 pipe: 13
+//    operations an increment (9 with plain sums).  A call of lbm_stats with them
+//    takes 84 us more than one without at 100^3 (11 separations), 1.74 ms at 400^3 (15), 3.42
+//    ms at 512^3 (16); 125 us, 3.34 and 7.03 ms with partners read from global memory.
+//  - k_struct_tiles<SUMS_EXACT>, for lbm_structure_functions_noalloc: the FP64 sums of
 //    the exact increments.  This part executes 2 FP64 operations per clock and
 //    SM against 128 in FP32, so increments, powers and running sums are kept as
 //    unevaluated sums of FP32 words (Dekker 1971; Knuth's two-sum, products with
 //    an FMA for the remainder).  Against quadruple-precision sums it is off by at most
 //    6e-16 of <|d|^p> for every p, on random, Taylor-Green, sinusoidal and ramp fields of
-//    7e4 to 1e6 cells (2e-16 typically), where the FP64 loop left 0.3-1.2e-14.  Each tile
+//    5e2 to 1e6 cells (2e-16 typically), where the FP64 loop left 0.1-1.2e-14.  Each tile
 //    scales its increments by a power of two so that neither the sixth power nor its low
 //    words leave the FP32 range; a tile whose values do not allow that (infinities, NaN,
 //    extreme exponents) is summed in FP64.  Bound by issue: ~215 FP32 operations an
@@ -50,12 +54,15 @@ constexpr int kCols = 32;       // pencils of a tile: one per lane
 constexpr int kPitch = 33;      // values between consecutive cells of a pencil
 constexpr int kRunMax = 64;     // cells a lane sums before the warp reduces
 constexpr int kRunMin = 4;      // fewer are not worth the reduction
+constexpr int64_t kSmallCells = 1 << 20;  // lattices up to 101^3: SUMS_1
 constexpr int kWarpsMax = 8;
 constexpr int kSmemMax = 225 * 1024;  // dynamic shared memory of a block, beside the few static words
 
-// Separations of one pass over a tile: its sums stay in registers (24 FP32 sums
+// Arithmetic of the sums: FP32 with plain sums of 4 cells, with none, or exact.
+enum { SUMS_4 = 0, SUMS_1 = 1, SUMS_EXACT = 2 };
+// Separations of one pass over a tile: its sums stay in registers (24 two-word sums
 // of 4 separations, or 12 three-word sums of 2).
-template <bool EXACT> constexpr int chunk_len() { return EXACT ? 2 : 4; }
+template <int SUMS> constexpr int chunk_len() { return SUMS == SUMS_EXACT ? 2 : 4; }
 
 __device__ __forceinline__ void stage4(uint32_t dst, const float* src, bool live) {
   // 4-byte asynchronous copy; a pencil past the end reads as zeros
@@ -118,21 +125,29 @@ struct PowerSums {
 };
 
 // Sum 24 values over the warp's 32 lanes, value i ending in lane i: each step
-// halves the values a lane holds (31 shuffles instead of 120).
-__device__ __forceinline__ float warp_sums(const float (&v)[24], int lane) {
-  float a[32];
+// halves the values a lane holds (31 additions instead of 120).  A value is h + l, l
+// of run_f32<K>; every remainder is kept, as FP64 additions (slow on this part) would.
+template <int K>
+__device__ __forceinline__ double warp_sums(const float (&h)[24], const float (&l)[24], int lane) {
+  float a[32], b[32];
 #pragma unroll
-  for (int i = 0; i < 32; ++i) a[i] = i < 24 ? v[i] : 0.f;
+  for (int i = 0; i < 32; ++i) {
+    a[i] = i < 24 ? h[i] : 0.f;
+    b[i] = i < 24 ? l[i] : 0.f;
+  }
 #pragma unroll
   for (int s = 16; s > 0; s >>= 1) {
     const bool up = (lane & s) != 0;
 #pragma unroll
     for (int i = 0; i < s; ++i) {
       const float send = up ? a[i] : a[i + s], keep = up ? a[i + s] : a[i];
-      a[i] = keep + __shfl_xor_sync(0xffffffffu, send, s);
+      float e, lo = 0.f;
+      a[i] = two_sum(keep, __shfl_xor_sync(0xffffffffu, send, s), e);
+      if (s < 16 || K == 1 || i % 2 == 0) lo = (up ? b[i + s] : b[i]) + __shfl_xor_sync(0xffffffffu, up ? b[i] : b[i + s], s);
+      b[i] = lo + e;
     }
   }
-  return a[0];
+  return (double)a[0] + (double)b[0];
 }
 
 // The same for the 12 three-word sums of two separations, value i ending in lanes
@@ -178,34 +193,82 @@ __device__ __forceinline__ Pair fma2(Pair a, Pair b, Pair c) {
   return r;
 }
 
-// Sums of one chunk over the run of n cells that starts at p (lane's pencil), FP32, two
-// separations to a register pair.
-__device__ __forceinline__ void run_f32(const float* p, const int (&off)[4], int n, float (&t)[24]) {
-  Pair s[2][6];
+// Plain FP32 sums span K cells; theirs, hi, keep what an addition rounds away in lo: of
+// the odd powers, whose terms cancel over a pencil but not within a run (neighbouring
+// increments are alike, so a running sum grows far beyond what is left of it), and with
+// K = 1 of the even ones too.  The remainder is exact while |hi| >= |s|, as it is after the
+// first of alike increments, and off by no more than the rounding of s itself otherwise.
+template <int K>
+struct PairSums {
+  Pair hi[2][6], lo[2][6];
+  static __device__ __forceinline__ constexpr bool keeps(int k) { return K == 1 || k % 2 == 0; }
+  __device__ __forceinline__ void reset() {
 #pragma unroll
-  for (int j = 0; j < 2; ++j)
+    for (int j = 0; j < 2; ++j)
 #pragma unroll
-    for (int k = 0; k < 6; ++k) s[j][k] = 0ull;
-#pragma unroll 8
-  for (int i = 0; i < n; ++i, p += kPitch) {
-    const float own = -p[0];
-    const Pair own2 = pack2(own, own);
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      const Pair d = add2(pack2(p[off[2 * j]], p[off[2 * j + 1]]), own2);
-      const Pair q = mul2(d, d), c = mul2(q, d);
-      s[j][0] = add2(s[j][0], d);
-      s[j][1] = add2(s[j][1], q);
-      s[j][2] = fma2(q, d, s[j][2]);
-      s[j][3] = fma2(q, q, s[j][3]);
-      s[j][4] = fma2(c, q, s[j][4]);
-      s[j][5] = fma2(c, c, s[j][5]);
-    }
+      for (int k = 0; k < 6; ++k) hi[j][k] = lo[j][k] = 0ull;
   }
+  // The C cells from p on.
+  template <int C>
+  __device__ __forceinline__ void add(const float* p, const int (&off)[4]) {
+    const Pair minus = pack2(-1.f, -1.f);
+    Pair s[2][6];
+#pragma unroll
+    for (int i = 0; i < C; ++i, p += kPitch) {
+      const float own = -p[0];
+      const Pair own2 = pack2(own, own);
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        const Pair d = add2(pack2(p[off[2 * j]], p[off[2 * j + 1]]), own2);
+        const Pair q = mul2(d, d), c = mul2(q, d);
+        if (i == 0) {
+          s[j][0] = d;
+          s[j][1] = q;
+          s[j][2] = c;
+          s[j][3] = mul2(q, q);
+          s[j][4] = mul2(c, q);
+          s[j][5] = mul2(c, c);
+        } else {
+          s[j][0] = add2(s[j][0], d);
+          s[j][1] = add2(s[j][1], q);
+          s[j][2] = fma2(q, d, s[j][2]);
+          s[j][3] = fma2(q, q, s[j][3]);
+          s[j][4] = fma2(c, q, s[j][4]);
+          s[j][5] = fma2(c, c, s[j][5]);
+        }
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+#pragma unroll
+      for (int k = 0; k < 6; ++k) {
+        const Pair t = add2(hi[j][k], s[j][k]);
+        if (keeps(k)) lo[j][k] = add2(lo[j][k], fma2(fma2(hi[j][k], minus, t), minus, s[j][k]));
+        hi[j][k] = t;
+      }
+  }
+};
+
+// Sums h + l of one chunk over the run of n cells that starts at p (lane's pencil), two
+// separations to a register pair.
+template <int K>
+__device__ __forceinline__ void run_f32(const float* p, const int (&off)[4], int n, float (&h)[24], float (&l)[24]) {
+  PairSums<K> t;
+  t.reset();
+#pragma unroll (8 / K)
+  for (int g = n / K; g > 0; --g, p += K * kPitch) t.template add<K>(p, off);
+  for (int i = n % K; i > 0; --i, p += kPitch) t.template add<1>(p, off);
 #pragma unroll
   for (int j = 0; j < 2; ++j)
 #pragma unroll
-    for (int k = 0; k < 6; ++k) unpack2(s[j][k], t[12 * j + k], t[12 * j + 6 + k]);
+    for (int k = 0; k < 6; ++k) {
+      unpack2(t.hi[j][k], h[12 * j + k], h[12 * j + 6 + k]);
+      if (PairSums<K>::keeps(k)) {
+        unpack2(t.lo[j][k], l[12 * j + k], l[12 * j + 6 + k]);
+      } else {
+        l[12 * j + k] = l[12 * j + 6 + k] = 0.f;
+      }
+    }
 }
 
 // The same in three-word arithmetic, increments times `scale` (a power of two).
@@ -258,12 +321,13 @@ __device__ __forceinline__ bool cells_differ(float a, float b) {
 
 // Tiles of the three axes in one numbering; a block takes tiles b, b + grid, ...
 // partials[block][nr][6].
-template <bool EXACT>
-__global__ void __launch_bounds__(kWarpsMax * 32, EXACT ? 2 : 3)
+template <int SUMS>
+__global__ void __launch_bounds__(kWarpsMax * 32, 2)
 k_struct_tiles(const float* __restrict__ u, StructPlan pl, double* __restrict__ partials) {
   extern __shared__ __align__(16) float tile[];  // [rows][33], then [warps][nr][6] doubles
   __shared__ float s_adj[kWarpsMax], s_top[kWarpsMax];
-  constexpr int CH = chunk_len<EXACT>();
+  constexpr bool EXACT = SUMS == SUMS_EXACT;
+  constexpr int CH = chunk_len<SUMS>();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
   const int nv = 6 * pl.nr;
   double* tot = reinterpret_cast<double*>(tile + pl.rows_max * kPitch);
@@ -360,11 +424,12 @@ k_struct_tiles(const float* __restrict__ u, StructPlan pl, double* __restrict__ 
         const int i = k0 * 6 + (lane >> 1);
         if (!(lane & 1) && lane < 24 && i < nv) mine[i] += v;
       } else {
-        float s[24];
-        run_f32(p, off, n, s);
-        const float v = warp_sums(s, lane);
+        float h[24], l[24];
+        constexpr int K = SUMS == SUMS_1 ? 1 : 4;
+        run_f32<K>(p, off, n, h, l);
+        const double v = warp_sums<K>(h, l, lane);
         const int i = k0 * 6 + lane;
-        if (lane < 24 && i < nv) mine[i] += (double)v;
+        if (lane < 24 && i < nv) mine[i] += v;
       }
     }
   }
@@ -431,12 +496,17 @@ __global__ void k_struct(const float* __restrict__ u, int nx, int ny, int nz, in
   }
 }
 
-template <bool EXACT>
-cudaError_t finish_plan(StructPlan& pl, int max_blocks, int sms) {
-  cudaError_t e = cudaFuncSetAttribute(k_struct_tiles<EXACT>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
+using TilesFn = void (*)(const float*, StructPlan, double*);
+TilesFn tiles_fn(const StructPlan& pl, bool exact) {
+  if (exact) return k_struct_tiles<SUMS_EXACT>;
+  return pl.ncell <= kSmallCells ? k_struct_tiles<SUMS_1> : k_struct_tiles<SUMS_4>;
+}
+
+cudaError_t finish_plan(StructPlan& pl, bool exact, int max_blocks, int sms) {
+  const TilesFn fn = tiles_fn(pl, exact);
+  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
   int per_sm = 0;
-  if (e == cudaSuccess)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_struct_tiles<EXACT>, pl.threads, pl.smem);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, pl.threads, pl.smem);
   if (e == cudaSuccess && per_sm < 1) e = cudaErrorInvalidConfiguration;
   if (e == cudaSuccess)
     pl.grid = (int)std::max<int64_t>(1, std::min<int64_t>({pl.tiles, (int64_t)per_sm * sms, (int64_t)max_blocks}));
@@ -507,14 +577,13 @@ bool plan_struct(int nx, int ny, int nz, const int* r, int nr, bool exact, int m
   // Shorter segments give every SM one.
   if (exact) smem = cut(sms);
   pl.smem = (int)smem;
-  *err = exact ? finish_plan<true>(pl, max_blocks, sms) : finish_plan<false>(pl, max_blocks, sms);
+  *err = finish_plan(pl, exact, max_blocks, sms);
   *out = pl;
   return *err == cudaSuccess;
 }
 
 cudaError_t launch_struct_plan(const float* u, const StructPlan& pl, bool exact, double* partials, cudaStream_t st) {
-  return exact ? launch_kernel(k_struct_tiles<true>, pl.grid, pl.threads, pl.smem, st, u, pl, partials)
-               : launch_kernel(k_struct_tiles<false>, pl.grid, pl.threads, pl.smem, st, u, pl, partials);
+  return launch_kernel(tiles_fn(pl, exact), pl.grid, pl.threads, pl.smem, st, u, pl, partials);
 }
 
 cudaError_t launch_struct(const float* u, int nx, int ny, int nz, int r, double* partials,
