@@ -1,4 +1,5 @@
-"""Benchmark of the GB300 MRT-Smagorinsky LBM step (one JSON line on stdout).
+"""Benchmark of the GB300 MRT-Smagorinsky LBM step (one JSON line on stdout; the extra
+workloads of a default run as one JSON line on stderr).
 
 Workload (headline): the forced-HIT DNS shape, an 800^3 periodic lattice
 (5.12e8 cells) with FP32 storage, seeded random solenoidal initial field
@@ -39,6 +40,14 @@ sys.path.insert(0, ROOT)
 BYTES_PER_UPDATE = {0: 152, 1: 76, 2: 76}  # 19 loads + 19 stores of one stored population
 DTYPE_NAME = {0: "f32", 1: "f32 (f16 storage)", 2: "f32 (bf16 storage)"}
 U0, CF, RE = 0.043, 0.2, 2.0e4
+
+
+def print_result(line, extra):
+    """The result as one JSON line on stdout; the extra workloads (spectra among them, tens of
+    kilobytes) as one on stderr, so that the end of a run's output holds the result whole."""
+    if extra:
+        print(json.dumps({"extra": extra}), file=sys.stderr, flush=True)
+    print(json.dumps(line), flush=True)
 
 
 def dist_env():
@@ -989,9 +998,8 @@ def main():
                             "(lbm_init_velocity_f32) + lbm_step(K) + lbm_stats"},
             "gpu_launches": args.steps,
             "clocks": clocks.summary(),
-            "extra": extra,
         }
-        print(json.dumps(line), flush=True)
+        print_result(line, extra)
     if dist:
         torch.distributed.destroy_process_group()
     return 0
