@@ -20,7 +20,7 @@
 //    time to spare: no plain sums at all.  Two separations share a register pair (f32x2
 //    operations).  Against FP64 sums of random solenoidal fields S_1 to S_6 are off by
 //    2e-11 to 6e-10 of <|d|^p> at 100^3 and 7e-12 to 2e-9 at 404^3; plain sums of 64 cells
-//    and the warp left S_1, S_3 and S_5 3-18 times that.  Bound by the FP32 pipe: 13
+//    and the warp left S_1, S_3 and S_5 2-20 times that.  Bound by the FP32 pipe: 13
 //    operations an increment (9 with plain sums).  A call of lbm_stats with them
 //    takes 84 us more than one without at 100^3 (11 separations), 1.74 ms at 400^3 (15), 3.42
 //    ms at 512^3 (16); 125 us, 3.34 and 7.03 ms with partners read from global memory.
@@ -39,6 +39,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cfloat>
 #include <climits>
 
 #include "lbm_check.cuh"
@@ -147,7 +148,8 @@ __device__ __forceinline__ double warp_sums(const float (&h)[24], const float (&
       b[i] = lo + e;
     }
   }
-  return (double)a[0] + (double)b[0];
+  // a sum that has left the FP32 range is infinite (or NaN), its remainder NaN
+  return fabsf(a[0]) <= FLT_MAX ? (double)a[0] + (double)b[0] : (double)a[0];
 }
 
 // The same for the 12 three-word sums of two separations, value i ending in lanes
