@@ -289,8 +289,9 @@ int lbm_energy_balance(const lbm_record_t* rec, int32_t n, double* residual, int
 
 /* Energy spectrum E(s), s = 0..kmax, of Eq. (integral_length_scale) with
  * |u_hat|^2, u_hat = N^-3 sum_x u exp(-2 pi i k.x/N), integer shells
- * s - 1/2 <= |k| < s + 1/2 (FP32 transform, shell sums in FP64; extents with prime
- * factors above 13 by cuFFT).  E points
+ * s - 1/2 <= |k| < s + 1/2 (FP32 transform; what a line of modes adds to a shell is
+ * rounded to FP32, shells are summed in FP64; extents with prime factors above 13 by
+ * cuFFT).  E points
  * to kmax + 1 doubles of host memory.  Synchronous.  Errors: INVALID_ARG
  * (kmax < 0), CUDA (cuFFT failures included). */
 int lbm_spectrum(lbm_t h, int32_t inst, double* E, int32_t kmax);

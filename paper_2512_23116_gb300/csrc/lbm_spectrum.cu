@@ -38,6 +38,7 @@
 #include "lbm_check.cuh"
 #include "lbm_kernels.h"
 #include "lbm_spectrum.h"
+#include "lbm_words.cuh"
 
 namespace lbm {
 
@@ -314,7 +315,9 @@ struct ShellTile {
 // + g L of line col with the energies e(i).  sqrt(p + k^2) grows by less than one
 // per mode, so a line's shells follow one another without a gap: the running sum of the
 // current shell is simply stored at its place.  A shell that began in the run of
-// the thread before goes through `carry`.  Ends without a barrier.
+// the thread before goes through `carry`.  Sums keep their remainders: what a line
+// gives a shell is rounded to FP32 once where it is stored (and once more with a
+// carry), the lines of a tile add up in two words.  Ends without a barrier.
 template <int W, int L, typename E>
 __device__ __forceinline__ void add_shells(const E& e, int k0, int nk, int per, int col, int g, int groups, const int* lp,
                                            const float* lw, const ShellTile<W>& t, int kmax, double* shells) {
@@ -325,26 +328,28 @@ __device__ __forceinline__ void add_shells(const E& e, int k0, int nk, int per, 
     int K = p + kb * kb, s = shell_of(K), top = s * s + s;
     bool first = kb > k0 && shell_of(K - 2 * kb + 1) == s;
     if (first) at = s - base;
-    float run = 0.f, held = 0.f;
+    float run = 0.f, low = 0.f, held = 0.f;
     float* r = t.run + (s - base) * (W + 1) + col;
 #pragma unroll
     for (int i = 0; i < L; ++i) {
       const int k = kb + i;
       if (k < ke) {
         if (K > top) {
-          if (first) held = run;
+          if (first) held = run + low;
           first = false;
-          run = 0.f;
+          run = low = 0.f;
           ++s;
           top += 2 * s;
           r += W + 1;
         }
-        run += e(i);
-        if (!first) *r = run;
+        float err;
+        run = two_sum(run, e(i), err);
+        low += err;
+        if (!first) *r = run + low;
         K += 2 * k + 1;
       }
     }
-    t.carry[g * W + col] = first ? run : held;
+    t.carry[g * W + col] = first ? run + low : held;
   }
   t.carry_at[g * W + col] = at;
   if (g == 0) {
@@ -354,9 +359,12 @@ __device__ __forceinline__ void add_shells(const E& e, int k0, int nk, int per, 
   __syncthreads();
   // carries: the first of those that go to one shell adds them all
   if (at >= 0 && (g == 1 || t.carry_at[(g - 1) * W + col] != at)) {
-    float v = t.carry[g * W + col];
-    for (int h = g + 1; h < groups && t.carry_at[h * W + col] == at; ++h) v += t.carry[h * W + col];
-    t.run[at * (W + 1) + col] += v;
+    float v = t.carry[g * W + col], low = 0.f, err;
+    for (int h = g + 1; h < groups && t.carry_at[h * W + col] == at; ++h) {
+      v = two_sum(v, t.carry[h * W + col], err);
+      low += err;
+    }
+    t.run[at * (W + 1) + col] += v + low;
   }
   __syncthreads();
   int s0 = INT32_MAX, s1 = -1;
@@ -367,11 +375,14 @@ __device__ __forceinline__ void add_shells(const E& e, int k0, int nk, int per, 
   }
   s1 = min(s1, kmax);
   for (int s = s0 + (int)threadIdx.x; s <= s1; s += blockDim.x) {
-    float acc = 0.f;
+    float acc = 0.f, low = 0.f, err;
 #pragma unroll
     for (int c = 0; c < W; ++c)
-      if (s >= t.first[c] && s <= t.last[c]) acc = fmaf(lw[c], t.run[(s - t.first[c]) * (W + 1) + c], acc);
-    shells[s] += (double)acc;
+      if (s >= t.first[c] && s <= t.last[c]) {
+        acc = two_sum(acc, lw[c] * t.run[(s - t.first[c]) * (W + 1) + c], err);  // lw is 0, 1 or 2: exact
+        low += err;
+      }
+    shells[s] += (double)acc + (double)low;
   }
 }
 
