@@ -310,6 +310,21 @@ void touch_pages(void* p, size_t bytes) {
   for (std::thread& t : pool) t.join();
 }
 
+// Copy n FP32 values of the device, widened there, straight into the caller's FP64 array.
+int fetch_widened(lbm_t h, const float* src, double* dst, int64_t n) {
+  const int64_t chunk = std::min<int64_t>(n, kChunkCells);
+  const int rc = ensure_scratch(h, sizeof(double) * (size_t)chunk);
+  if (rc != LBM_OK) return rc;
+  touch_pages(dst, sizeof(double) * (size_t)n);
+  double* s = static_cast<double*>(h->d_scratch);
+  for (int64_t c0 = 0; c0 < n; c0 += chunk) {
+    const int64_t m = std::min(chunk, n - c0);
+    CK(h, launch_widen(src + c0, m, s, h->stream));
+    CK(h, cudaMemcpyAsync(dst + c0, s, sizeof(double) * m, cudaMemcpyDeviceToHost, h->stream));
+  }
+  return LBM_OK;
+}
+
 void clear_graphs(lbm_t h) {
   for (auto& kv : h->graphs) cudaGraphExecDestroy(kv.second);
   h->graphs.clear();
@@ -1660,23 +1675,10 @@ LBM_API int lbm_get_fields(lbm_t h, int32_t inst, double* drho, double* u, doubl
   Inst& I = h->inst[inst];
   int rc = diag_pass(h, inst, u != nullptr, drho || snorm || theta, -1, 0, false);
   if (rc != LBM_OK) return rc;
-  // widened on the device, copied straight into the caller's array
-  const int64_t chunk = std::min<int64_t>(3 * I.ncell, kChunkCells);
-  if ((rc = ensure_scratch(h, sizeof(double) * (size_t)chunk)) != LBM_OK) return rc;
-  auto fetch = [&](const float* src, double* dst, int64_t n) -> int {
-    touch_pages(dst, sizeof(double) * (size_t)n);
-    double* s = static_cast<double*>(h->d_scratch);
-    for (int64_t c0 = 0; c0 < n; c0 += chunk) {
-      const int64_t m = std::min(chunk, n - c0);
-      CK(h, launch_widen(src + c0, m, s, h->stream));
-      CK(h, cudaMemcpyAsync(dst + c0, s, sizeof(double) * m, cudaMemcpyDeviceToHost, h->stream));
-    }
-    return LBM_OK;
-  };
-  if (u && (rc = fetch(I.u, u, 3 * I.ncell)) != LBM_OK) return rc;
-  if (drho && (rc = fetch(I.aux, drho, I.ncell)) != LBM_OK) return rc;
-  if (snorm && (rc = fetch(I.aux + I.ncell, snorm, I.ncell)) != LBM_OK) return rc;
-  if (theta && (rc = fetch(I.aux + 2 * I.ncell, theta, I.ncell)) != LBM_OK) return rc;
+  if (u && (rc = fetch_widened(h, I.u, u, 3 * I.ncell)) != LBM_OK) return rc;
+  if (drho && (rc = fetch_widened(h, I.aux, drho, I.ncell)) != LBM_OK) return rc;
+  if (snorm && (rc = fetch_widened(h, I.aux + I.ncell, snorm, I.ncell)) != LBM_OK) return rc;
+  if (theta && (rc = fetch_widened(h, I.aux + 2 * I.ncell, theta, I.ncell)) != LBM_OK) return rc;
   return check_err(h);
 }
 
@@ -1697,17 +1699,17 @@ LBM_API int lbm_get_theta_slice(lbm_t h, int32_t inst, int32_t axis, int32_t ind
   int rc = diag_pass(h, inst, false, false, axis, index, false);
   if (rc != LBM_OK) return rc;
   const size_t n = axis == 0 ? (size_t)p.nz * p.ny : (axis == 1 ? (size_t)p.nz * p.nx : (size_t)p.ny * p.nx);
-  const size_t chunk = std::min(n, kPinBytes / sizeof(float) - 1);  // larger planes in pieces
-  if ((rc = ensure_pin(h, sizeof(float) * (chunk + 1))) != LBM_OK) return rc;
-  float* buf = reinterpret_cast<float*>(h->pin);
-  uint32_t* err = reinterpret_cast<uint32_t*>(buf + chunk);
-  if ((rc = fetch_err(h, err)) != LBM_OK) return rc;
-  for (size_t c0 = 0; c0 < n; c0 += chunk) {
-    const size_t m = std::min(chunk, n - c0);
-    CK(h, cudaMemcpyAsync(buf, I.plane + c0, sizeof(float) * m, cudaMemcpyDeviceToHost, h->stream));
-    CK(h, cudaStreamSynchronize(h->stream));
-    for (size_t k = 0; k < m; ++k) host[c0 + k] = buf[k];
+  if (sizeof(float) * (n + 1) > kPinBytes) {  // 256^2 and larger: like the fields
+    if ((rc = fetch_widened(h, I.plane, host, (int64_t)n)) != LBM_OK) return rc;
+    return check_err(h);
   }
+  if ((rc = ensure_pin(h, sizeof(float) * (n + 1))) != LBM_OK) return rc;
+  float* buf = reinterpret_cast<float*>(h->pin);
+  uint32_t* err = reinterpret_cast<uint32_t*>(buf + n);
+  if ((rc = fetch_err(h, err)) != LBM_OK) return rc;
+  CK(h, cudaMemcpyAsync(buf, I.plane, sizeof(float) * n, cudaMemcpyDeviceToHost, h->stream));
+  CK(h, cudaStreamSynchronize(h->stream));
+  for (size_t k = 0; k < n; ++k) host[k] = buf[k];
   return report_err(h, *err);
 }
 
