@@ -101,8 +101,9 @@ typedef struct lbm_params {
   int32_t tile_rows;      /* rows (of nx cells) per tile of the TMA kernel; 0: autotune.  The
                              direct kernel deals out cells in chunks of a block */
   int32_t stages;         /* TMA pipeline stages; 0: autotune */
-  int32_t threads;        /* threads per block; 0: autotune.  kernel, tile_rows,
-                             stages (TMA) and threads all set: no autotuning */
+  int32_t threads;        /* threads per block; 0: autotune.  kernel and threads
+                             (TMA: tile_rows and stages too) all set: no
+                             autotuning.  The direct kernel takes up to 256 */
   int32_t row_align;      /* byte alignment of each x-line (power of two >= 16;
                              0: 16).  Padding costs memory, not bandwidth: only
                              the nx live cells of a line are moved */

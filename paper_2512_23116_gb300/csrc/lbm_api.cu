@@ -41,6 +41,7 @@ constexpr int kMinHistWindow = 256;  // fewer histogram bins than this in shared
 constexpr int64_t kChunkCells = 4 << 20;
 constexpr size_t kDirectBytes = 24 << 20;     // populations up to this size: direct kernel, no others timed
 constexpr size_t kDirectMaxBytes = 40 << 20;  // and up to this size (FP32): the direct kernel among others
+constexpr int kDirectThreads = 256;           // most threads of its blocks
 constexpr size_t kPinBytes = 256 << 10;       // page-locked staging of small results, at least
 constexpr size_t kFftBatchBytes = 192 << 20;  // three half spectra (256^3) transformed together
 constexpr double kPi = 3.14159265358979323846;
@@ -1071,8 +1072,9 @@ int choose_config(lbm_t h, const lbm_params& p0) {
   // means population-major otherwise
   const int lay_req = p0.layout;
   const int lay_fixed = lay_req == 2 ? 1 : 0;
-  // a fully specified configuration skips the autotuner
-  if (requested_kind == 1 && requested_rows > 0 && p0.threads > 0)
+  // a fully specified configuration skips the autotuner (the direct kernel's is its block
+  // size; without tile_rows one above its launch bound is left to the autotuner)
+  if (requested_kind == 1 && p0.threads > 0 && (requested_rows > 0 || p0.threads <= kDirectThreads))
     return apply_candidate(h, {1, p0.threads, 0, 0, requested_rows, 0, lay_fixed});
   const bool allow_slots = p0.tma_slots == 0;
   if (requested_kind == 2 && requested_rows > 0 && p0.threads > 0 && p0.stages > 0) {
@@ -1187,7 +1189,7 @@ int choose_config(lbm_t h, const lbm_params& p0) {
   Candidate bc = cands[0];
   for (const Candidate& c : cands) {
     if (apply_candidate(h, c) != LBM_OK) continue;
-    const double ms = time_candidate(h, steps, direct_only);
+    const double ms = time_candidate(h, steps, bytes <= kDirectBytes);
     if (ms < best) {
       best = ms;
       bc = c;
