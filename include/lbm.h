@@ -350,7 +350,8 @@ int lbm_device_ptr(lbm_t h, int32_t inst, void** ptr, size_t* bytes, int32_t* nx
 /* Effective parameters after derivation: nu0, s_nu0, F0, C of `inst`. */
 int lbm_get_params(lbm_t h, int32_t inst, double* nu0, double* s_nu0, double* f0, double* C);
 
-/* Kernel chosen by the autotuner: kind (1 direct, 2 TMA bulk), tile rows,
+/* Kernel chosen by the autotuner: kind (1 direct, 2 TMA bulk), tile rows (of
+ * the direct kernel, which has no tiles, those asked for; 0: none),
  * pipeline stages, threads per block, blocks per SM, population layout (1
  * population-major, 2 row-interleaved), shared-memory slot bytes of the TMA
  * tiles (0: runtime stride).  Any pointer may be NULL. */

@@ -344,21 +344,19 @@ int build_tiles(lbm_t h) {
   for (size_t i = 0; i < h->inst.size(); ++i) {
     Inst& I = h->inst[i];
     const lbm_params& p = I.p;
-    int R;
+    int R = std::min(h->rows_fixed, p.ny), tpp = 0;  // the direct kernel has no tiles: what was asked for is kept
     const int64_t row_bytes = (int64_t)19 * I.nxp * (int64_t)h->esize;
+    I.tile_begin = tile;
     if (h->kind == 2) {
       // a TMA stage holds at most tile_bytes_max bytes (19 segments of R x nxp values)
       const int64_t cap = h->tile_bytes_max / row_bytes;
       if (cap < 1) return fail(h, LBM_ERR_UNSUPPORTED, "an x-line of instance %zu does not fit a stage", i);
       R = (int)(h->rows_fixed > 0 ? std::min<int64_t>(h->rows_fixed, cap) : cap);
-    } else {
-      R = h->rows_fixed > 0 ? h->rows_fixed : std::max(1, (1024 + p.nx - 1) / p.nx);
+      R = std::max(1, std::min(R, p.ny));
+      tpp = (p.ny + R - 1) / R;
+      tile += (int64_t)tpp * p.nz;
     }
-    R = std::max(1, std::min(R, p.ny));
     I.rows = R;
-    const int tpp = (p.ny + R - 1) / R;
-    I.tile_begin = tile;
-    tile += (int64_t)tpp * p.nz;
     I.tile_end = tile;
     I.chunk_begin = chunk;
     chunk += (I.ncell + h->chunk - 1) / h->chunk;
@@ -585,7 +583,7 @@ int diag_pass(lbm_t h, int i, bool want_u, bool want_aux, int plane_axis, int pl
   // plane by plane), and no reduction of the block partials, which then
   // cover the plane only
   const bool plane_only = plane_axis == 2 && !want_u && !want_aux && !want_hist;
-  if (plane_only) {
+  if (plane_only && h->kind == 2) {
     const int64_t tpp = (I.p.ny + I.rows - 1) / I.rows;
     la.tile_lo = I.tile_begin + (int64_t)plane_index * tpp;
     la.tile_hi = la.tile_lo + tpp;
