@@ -164,19 +164,21 @@ __device__ __forceinline__ void stage(float2* s, const float2* tw, const FftAxis
   const int m = ax.m[i], count = m * done, dj = ax.dj[i], db = ax.db[i];
   int blk = (int)(((float)g + 0.5f) * ax.inv_m[i]), j = g - blk * m;
   for (int b = g; b < count; b += groups) {
-    float2* p = s + (blk * R * m + j) * P + col;
-    float2 x[R];
+    if (in_bounds(blk >= 0 && j >= 0 && blk * R * m + j + (R - 1) * m < ax.n && (R - 1) * j * done < ax.n)) {
+      float2* p = s + (blk * R * m + j) * P + col;
+      float2 x[R];
 #pragma unroll
-    for (int q = 0; q < R; ++q) x[q] = p[q * m * P];
-    Dft<R>::run(x);
-    p[0] = x[0];
-    if (m > 1) {
-      const int step = j * done;
+      for (int q = 0; q < R; ++q) x[q] = p[q * m * P];
+      Dft<R>::run(x);
+      p[0] = x[0];
+      if (m > 1) {
+        const int step = j * done;
 #pragma unroll
-      for (int q = 1; q < R; ++q) p[q * m * P] = cmul(x[q], tw[q * step]);
-    } else {
+        for (int q = 1; q < R; ++q) p[q * m * P] = cmul(x[q], tw[q * step]);
+      } else {
 #pragma unroll
-      for (int q = 1; q < R; ++q) p[q * P] = x[q];
+        for (int q = 1; q < R; ++q) p[q * P] = x[q];
+      }
     }
     j += dj;
     blk += db;
@@ -195,6 +197,7 @@ __device__ __forceinline__ void stage_prime(float2* s, const float2* tw, const F
   const int m = ax.m[i], count = m * done, n = ax.n;
   for (int b = g; b < count; b += groups) {
     const int blk = b / m, j = b - blk * m;
+    if (!in_bounds(blk * R * m + j + (R - 1) * m < n && (R - 1) * j * done < n)) continue;
     float2* p = s + (blk * R * m + j) * P + col;
     const float2 x0 = p[0];
     float2 t[R / 2], d[R / 2];
@@ -345,7 +348,7 @@ __device__ __forceinline__ void add_shells(const E& e, int k0, int nk, int per, 
         float err;
         run = two_sum(run, e(i), err);
         low += err;
-        if (!first) *r = run + low;
+        if (!first && in_bounds(s >= base && s - base < nk)) *r = run + low;
         K += 2 * k + 1;
       }
     }
@@ -358,7 +361,7 @@ __device__ __forceinline__ void add_shells(const E& e, int k0, int nk, int per, 
   }
   __syncthreads();
   // carries: the first of those that go to one shell adds them all
-  if (at >= 0 && (g == 1 || t.carry_at[(g - 1) * W + col] != at)) {
+  if (at >= 0 && in_bounds(at < nk) && (g == 1 || t.carry_at[(g - 1) * W + col] != at)) {
     float v = t.carry[g * W + col], low = 0.f, err;
     for (int h = g + 1; h < groups && t.carry_at[h * W + col] == at; ++h) {
       v = two_sum(v, t.carry[h * W + col], err);
@@ -378,7 +381,7 @@ __device__ __forceinline__ void add_shells(const E& e, int k0, int nk, int per, 
     float acc = 0.f, low = 0.f, err;
 #pragma unroll
     for (int c = 0; c < W; ++c)
-      if (s >= t.first[c] && s <= t.last[c]) {
+      if (s >= t.first[c] && s <= t.last[c] && in_bounds(s - t.first[c] < nk)) {
         acc = two_sum(acc, lw[c] * t.run[(s - t.first[c]) * (W + 1) + c], err);  // lw is 0, 1 or 2: exact
         low += err;
       }
@@ -413,7 +416,8 @@ __global__ void __launch_bounds__(kFftThreads, PRIMES ? 1 : 2) k_fft_pass(FftArg
   const int tid = threadIdx.x, col = tid % W, g = tid / W, groups = blockDim.x / W;
   for (int k = tid; k < n; k += blockDim.x) {
     tw[k] = a.tw[k];
-    row[k] = (uint16_t)row_of(a.ax, k);
+    const int r = row_of(a.ax, k);
+    row[k] = (uint16_t)(in_bounds(r >= 0 && r < n) ? r : 0);
   }
   if (PASS == PASS_X)
     for (int k = tid; k <= a.kmax; k += blockDim.x) shells[k] = 0.0;

@@ -179,7 +179,9 @@ k_step_direct(const InstDesc* __restrict__ insts, int ninst, int64_t chunk_lo, i
 #pragma unroll
       for (int a = 0; a < 19; ++a)
         f[a] = in_bounds((int64_t)o[a] >= 0 && (int64_t)o[a] < (ONE ? one : insts[cur]).f_elems) ? S::load(fb + o[a]) : 0.f;
-      const float Fx = fx[w.y] + cfx, Fy = fy[w.z] + cfy, Fz = fz[w.x] + cfz;
+      const bool cell_ok = in_bounds(w.x >= 0 && w.x < w.nx && w.y >= 0 && w.y < w.ny && w.z >= 0 && w.z < w.nz);
+      const float Fx = (cell_ok ? fx[w.y] : 0.f) + cfx, Fy = (cell_ok ? fy[w.z] : 0.f) + cfy,
+                  Fz = (cell_ok ? fz[w.x] : 0.f) + cfz;
       CellDiag g;
       mrt_collide(f, Fx, Fy, Fz, nu0, s_nu0, C, g, decltype(mode)::value);
       if (MODE != MODE_DIAG) {

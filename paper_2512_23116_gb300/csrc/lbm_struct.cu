@@ -402,12 +402,16 @@ k_struct_tiles(const float* __restrict__ u, StructPlan pl, double* __restrict__ 
       kexp = tile_exponent(adj, top);
     }
     const int q = (len + nwarps - 1) / nwarps;
-    const int n = max(0, min(q, len - warp * q));
+    int n = max(0, min(q, len - warp * q));
+    if (!in_bounds(n == 0 || (warp * q + n + ax.halo <= rows && rows <= pl.rows_max))) n = 0;
     const float* p = tile + warp * q * kPitch + lane;
     for (int k0 = 0; k0 < pl.nr; k0 += CH) {
       int off[CH];  // a chunk past the last separation is padded with r = 0: zero increments
 #pragma unroll
-      for (int j = 0; j < CH; ++j) off[j] = (k0 + j < pl.nr ? pl.r[a][k0 + j] : 0) * kPitch;
+      for (int j = 0; j < CH; ++j) {
+        const int r = k0 + j < pl.nr ? pl.r[a][k0 + j] : 0;
+        off[j] = (in_bounds(r >= 0 && r <= ax.halo) ? r : 0) * kPitch;
+      }
       if constexpr (EXACT) {
         double v;
         if (kexp == INT_MIN) {
