@@ -117,7 +117,9 @@ __device__ __forceinline__ float strain_norm(float TT, float Qt, float nu0, floa
   const float b = 0.5f + 3.f * nu0;
   const float p2 = 2.f * TT;
   const float p = p2 > 1e-30f ? p2 * rsqrtf(p2) : 0.f;
-  const float q = b * b + 12.f * C * p;  // >= b^2 >= 1/4
+  // b^2 rounded first, spelled out: left to the compiler, the step of the direct kernel
+  // rounded 12 C p first and its populations differed from the TMA kernel's in the last bit
+  const float q = fmaf(12.f * C, p, __fmul_rn(b, b));  // >= b^2 >= 1/4
   const float xs = __fdividef(2.f * p, b + q * rsqrtf(q));
   const float x2 = xs * xs + 2.f * Qt;
   float x = x2 > 1e-30f ? x2 * rsqrtf(x2) : 0.f;
