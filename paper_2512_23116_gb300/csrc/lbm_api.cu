@@ -1097,15 +1097,8 @@ int choose_config(lbm_t h, const lbm_params& p0) {
   // against 20.3) and the TMA kernel is ahead once it is shared or outgrown (three
   // lattices of 100^3 stepped in turn: 22.8 against 27.5 us; three of 96^3 in FP16, 34 MB
   // each: 9.0 against 10.0).
-  // The two kernels give the same bits but for the self-consistent strain (strain_mode 1),
-  // whose last bit differs; in 16-bit storage that grows to a spacing of the storage
-  // format, so such handles stay with the TMA kernel whatever their size.
-  bool alike = h->precision == LBM_FP32;
-  if (!alike) {
-    alike = true;
-    for (const Inst& I : h->inst) alike = alike && I.p.strain_mode == 0;
-  }
-  const bool direct_only = requested_kind == 0 && alike && bytes <= kDirectBytes;
+  // The two kernels give the same bits.
+  const bool direct_only = requested_kind == 0 && bytes <= kDirectBytes;
   const bool want_direct =
       requested_kind == 1 || (requested_kind == 0 && (direct_only || (h->precision == LBM_FP32 && bytes <= kDirectMaxBytes) || !tma_ok));
   if (want_direct)
