@@ -42,6 +42,7 @@ constexpr int64_t kChunkCells = 4 << 20;
 constexpr size_t kDirectBytes = 24 << 20;     // populations up to this size: direct kernel, no others timed
 constexpr size_t kDirectMaxBytes = 40 << 20;  // and up to this size (FP32): the direct kernel among others
 constexpr int kDirectThreads = 256;           // most threads of its blocks
+constexpr int64_t kSmallPlane = 700;          // and with fewer cells a plane than this: both at any size
 constexpr size_t kPinBytes = 256 << 10;       // page-locked staging of small results, at least
 constexpr size_t kFftBatchBytes = 192 << 20;  // three half spectra (256^3) transformed together
 constexpr double kPi = 3.14159265358979323846;
@@ -1088,7 +1089,12 @@ int choose_config(lbm_t h, const lbm_params& p0) {
     return apply_candidate(h, c);
   }
   size_t bytes = 0;
-  for (const Inst& I : h->inst) bytes += I.f_bytes;
+  int64_t cells = 0, planes = 0;
+  for (const Inst& I : h->inst) {
+    bytes += I.f_bytes;
+    cells += I.ncell;
+    planes += I.p.nz;
+  }
   // Lattices deep inside the L2 cache always step fastest with the direct kernel (a TMA
   // block sees a tile or two per step, all of it pipeline fill and drain): FP32 32^3
   // 2.1 against 5.1 us, 64^3 (20 MB) 6.1 against 8.6; FP16 80^3 (19 MB) 9.7 against 11.4.
@@ -1097,10 +1103,16 @@ int choose_config(lbm_t h, const lbm_params& p0) {
   // against 20.3) and the TMA kernel is ahead once it is shared or outgrown (three
   // lattices of 100^3 stepped in turn: 22.8 against 27.5 us; three of 96^3 in FP16, 34 MB
   // each: 9.0 against 10.0).
+  // Where planes are small the two are timed at any size: a TMA tile never crosses a plane,
+  // and the copies of one of a few hundred cells take as long as those of the 700 cells
+  // it has at 100^3.  8 x 8 x 30000 steps in 54 against 224 us, 16 x 16 x 8000 in 59 against
+  // 73, 24 x 24 x 3000 (576 cells a plane) in 47 either way, in FP16 in 29 against 34.
   // The two kernels give the same bits.
   const bool direct_only = requested_kind == 0 && bytes <= kDirectBytes;
+  const bool small_planes = cells < kSmallPlane * planes;
   const bool want_direct =
-      requested_kind == 1 || (requested_kind == 0 && (direct_only || (h->precision == LBM_FP32 && bytes <= kDirectMaxBytes) || !tma_ok));
+      requested_kind == 1 || (requested_kind == 0 && (direct_only || (h->precision == LBM_FP32 && bytes <= kDirectMaxBytes) ||
+                                                      small_planes || !tma_ok));
   if (want_direct)
     for (int th : {64, 128, 256}) cands.push_back({1, th, 0, 0, requested_rows, 0, lay_fixed});
   if ((requested_kind == 2 || requested_kind == 0) && !direct_only && tma_ok) {
@@ -1172,15 +1184,15 @@ int choose_config(lbm_t h, const lbm_params& p0) {
   if (cands.empty())
     return fail(h, LBM_ERR_UNSUPPORTED, "no kernel configuration fits this lattice");
   if (cands.size() == 1) return apply_candidate(h, cands[0]);
-  // time each candidate on the rest state
-  int64_t cells = 0;
-  for (const Inst& I : h->inst) cells += I.ncell;
+  // time each candidate on the rest state; beyond the sizes above the direct kernel has to
+  // be ahead by 5 %, for the cache that it needs may be shared
+  const bool large = requested_kind == 0 && bytes > (h->precision == LBM_FP32 ? kDirectMaxBytes : kDirectBytes);
   const int steps = cells > (int64_t)64 << 20 ? 2 : (cells > (int64_t)4 << 20 ? 4 : 8);
   double best = 1e300;
   Candidate bc = cands[0];
   for (const Candidate& c : cands) {
     if (apply_candidate(h, c) != LBM_OK) continue;
-    const double ms = time_candidate(h, steps, bytes <= kDirectBytes);
+    const double ms = time_candidate(h, steps, bytes <= kDirectBytes) * (c.kind == 1 && large ? 1.05 : 1.0);
     if (ms < best) {
       best = ms;
       bc = c;
