@@ -354,11 +354,4 @@ __device__ __forceinline__ int find_instance(const InstDesc* __restrict__ insts,
   return i;
 }
 
-// The same for the direct kernel's chunks.
-__device__ __forceinline__ int find_chunk_instance(const InstDesc* __restrict__ insts, int ninst, int64_t t, int hint) {
-  int i = hint;
-  while (i + 1 < ninst && t >= insts[i].chunk_end) ++i;
-  return i;
-}
-
 }  // namespace lbm
