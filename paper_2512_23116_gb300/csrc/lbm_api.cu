@@ -44,7 +44,7 @@ constexpr size_t kDirectMaxBytes = 40 << 20;  // and up to this size (FP32): the
 constexpr int kDirectThreads = 256;           // most threads of its blocks
 constexpr int64_t kSmallPlane = 700;          // and with fewer cells a plane than this: both at any size
 constexpr size_t kPinBytes = 256 << 10;       // page-locked staging of small results, at least
-constexpr size_t kFftBatchBytes = 192 << 20;  // three half spectra (256^3) transformed together
+constexpr size_t kFftBatchBytes = 192 << 20;  // three half spectra (up to 255^3) transformed together
 constexpr double kPi = 3.14159265358979323846;
 
 thread_local std::string g_create_error;
@@ -1097,16 +1097,17 @@ int choose_config(lbm_t h, const lbm_params& p0) {
   }
   // Lattices deep inside the L2 cache always step fastest with the direct kernel (a TMA
   // block sees a tile or two per step, all of it pipeline fill and drain): FP32 32^3
-  // 2.1 against 5.1 us, 64^3 (20 MB) 6.1 against 8.6; FP16 80^3 (19 MB) 9.7 against 11.4.
-  // In FP32 both are timed up to kDirectMaxBytes (80^3, 39 MB: 10.6 against 12.5); above,
+  // 2.1 against 5.2 us, 64^3 (20 MB) 6.2 against 8.6; FP16 80^3 (19 MB) 9.7 against 11.4.
+  // In FP32 both are timed up to kDirectMaxBytes (80^3, 39 MB: 10.5 against 12.4); above,
   // the two are level while the cache is the lattice's own (100^3, 76 MB: 19.9
   // against 20.3) and the TMA kernel is ahead once it is shared or outgrown (three
   // lattices of 100^3 stepped in turn: 22.8 against 27.5 us; three of 96^3 in FP16, 34 MB
   // each: 9.0 against 10.0).
   // Where planes are small the two are timed at any size: a TMA tile never crosses a plane,
   // and the copies of one of a few hundred cells take as long as those of the 700 cells
-  // it has at 100^3.  8 x 8 x 30000 steps in 54 against 224 us, 16 x 16 x 8000 in 59 against
-  // 73, 24 x 24 x 3000 (576 cells a plane) in 47 either way, in FP16 in 29 against 34.
+  // it has at 100^3.  Direct against TMA: 8 x 8 x 30000 54 and 224 us a step, 16 x 16 x 8000
+  // 59 and 73, 24 x 24 x 3000 (576 cells a plane) 50 and 47, in FP16 29 and 34, 26 x 26 x 2600 56
+  // either way and 30 and 34, 32 x 32 x 2000 60 and 55, 37 and 33.
   // The two kernels give the same bits.
   const bool direct_only = requested_kind == 0 && bytes <= kDirectBytes;
   const bool small_planes = cells < kSmallPlane * planes;

@@ -6,7 +6,7 @@
 // adds its modes to the shells straight from shared memory instead of writing
 // them.  20 bytes of traffic per cell and component; the library's transform
 // followed by a binning pass moves 28.  Three components, transform and shells:
-// 100^3 73 -> 37 us, 400^3 3.68 -> 1.37 ms, 800^3 37.6 -> 11.4 ms.  A pass is bound
+// 100^3 73 -> 38 us, 400^3 3.68 -> 1.40 ms, 800^3 37.6 -> 11.6 ms.  A pass is bound
 // by issue (67 % of the issue slots at 320^3: ~90 instructions a point, two thirds of them the
 // stages) with its DRAM traffic at 60 % of the copy bandwidth.
 //

@@ -14,14 +14,13 @@
 // 32-bit for arrays below 4 GB (WIDE = false).
 //
 // What bounds it: the L2 cache.  With the collision taken out a step of 64^3 takes
-// 5.7 of its 6.1 us and one of 100^3 18.5 of 19.9 (9 TB/s; the odd step's x-shifted
+// 5.7 of its 6.2 us and one of 100^3 18.5 of 19.9 (9 TB/s; the odd step's x-shifted
 // slots cost 2-3 us of that in partly written sectors); prefetching the next
 // cell, into registers or by asynchronous copies, made it slower.  Below that it is
 // latency: launches and the first loads, which the launch parameter `one`, 32-bit
-// divisions and dependent launches shorten.  A step of 16^3 1.5 us, 32^3 2.1 (5.1 before,
-// the TMA kernel's; 5.8 for one-thread-per-cell tiles of whole rows with 64-bit offsets),
-// 48^3 3.5 (6.0), 64^3 6.1 (8.6), 80^3 10.6 (12.5); beyond ~100^3 the TMA kernel is ahead
-// (128^3: 54 against 61).
+// divisions and dependent launches shorten.  A step of 16^3 takes 1.5 us, 32^3 2.1 (the TMA
+// kernel 5.2), 48^3 3.7 (6.2), 64^3 6.2 (8.6), 80^3 10.5 (12.4); beyond ~100^3 the TMA
+// kernel is ahead (128^3: 54 against 61), but for boxes of small planes.
 #include <cuda_runtime.h>
 
 #include <type_traits>

@@ -35,7 +35,7 @@
 //    words leave the FP32 range; a tile whose values do not allow that (infinities, NaN,
 //    extreme exponents) is summed in FP64.  Bound by issue: ~215 FP32 operations an
 //    increment.  12 separations at 160^3: 4.50 ms (one FP64 pass over global memory
-//    per separation, at the FP64 rate) -> 1.14 ms.
+//    per separation, at the FP64 rate) -> 1.15 ms.
 #include <cuda_runtime.h>
 
 #include <algorithm>

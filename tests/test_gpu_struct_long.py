@@ -34,7 +34,7 @@ def _device_time(lbm, shape, seps):
 
 
 def test_a_long_box_takes_no_longer_than_its_cells_need(gpu_lib):
-    """8,000 cells either way; 4 tiles on 4 SMs took 10 and more times the cube's time.  The
-    long box stages more halo: 3 times is allowed."""
+    """8,000 cells either way.  The long box stages more halo and takes 2.3 times as long; in 4
+    tiles on 4 SMs it took 23 times.  The line lies between, far from the noise."""
     seps = list(range(1, 25))
-    assert _device_time(gpu_lib, (2, 2, 2000), seps) <= 3 * _device_time(gpu_lib, (20, 20, 20), seps)
+    assert _device_time(gpu_lib, (2, 2, 2000), seps) <= 7 * _device_time(gpu_lib, (20, 20, 20), seps)
